@@ -69,21 +69,15 @@ extern "C" {
 #define GVM_SGEMM_FMA 0    /* binary32 fused multiply-add on the CUDA cores */
 #define GVM_SGEMM_SPLIT3 1 /* A = Ah + Al, B = Bh + Bl in bf16; C = AhBh + AhBl + AlBh on
                               tcgen05 tensor cores with binary32 accumulation in TMEM.
-                              The manager splits while staging operands into shared
-                              memory (no scratch); gvm_sgemm_f32 runs a split pre-pass
-                              into caller scratch, then TMA-fed GEMM tiles */
-#define GVM_SGEMM_SPLIT3_FUSED 2 /* gvm_sgemm_f32 only: the manager's form of split3 (split
-                              during staging, no scratch); bit-identical to
-                              GVM_SGEMM_SPLIT3 */
+                              Operands are split while they are staged into shared memory.
+                              One kernel (256 x 256 tiles of a cluster of two CTAs) serves
+                              this and the three values below, which named other tile forms
+                              with the same results; gvm_sgemm_f32 still asks for scratch
+                              with this value */
+#define GVM_SGEMM_SPLIT3_FUSED 2 /* gvm_sgemm_f32 only: split3 without scratch */
 /* 3 is not used (it named a removed form); gvm_sgemm_f32 refuses it. */
-#define GVM_SGEMM_SPLIT3_WIDE 4 /* split during staging on 256 x 256 tiles of one CTA (the
-                              two 128-row halves share each B stage; one accumulator);
-                              bit-identical to GVM_SGEMM_SPLIT3. Also a manager path */
-#define GVM_SGEMM_SPLIT3_TMA 5 /* manager path only: 128 x 256 tiles whose binary32 A and B
-                              arrive by TMA boxes (a tensor map of each per task, where A
-                              and B are 16-byte aligned with row pitches of 16-byte
-                              multiples; other tasks are loaded by the converting warps)
-                              and are split in place; bit-identical to GVM_SGEMM_SPLIT3 */
+#define GVM_SGEMM_SPLIT3_WIDE 4 /* split3 (gvm_sgemm_f32: without scratch). Also a manager path */
+#define GVM_SGEMM_SPLIT3_TMA 5 /* split3, manager path only */
 
 /* ---- manager modes ------------------------------------------------------ */
 #define GVM_MODE_BARRIER 0    /* Section 5 request barrier: gvm_flush runs the scheduler
@@ -137,7 +131,8 @@ typedef struct gvm_config {
                                host wait in gvm_sync / gvm_wait_idle; 0 = 10 s */
   uint64_t idle_poll_ns;    /* sleep of an idle scheduler CTA between polls of the
                                rings; 0 = 1000 ns */
-  int32_t grid_ctas;        /* scheduler CTAs; 0 = one per SM */
+  int32_t grid_ctas;        /* scheduler CTAs; 0 = one per SM (two on the FMA path). The split3
+                               scheduler runs in pairs of CTAs: an odd number is rounded up */
   int32_t ingest_quantum;   /* tasks taken from one rank per ingest pass; 0 = 4 */
   uint64_t copy_run_bytes;  /* host-mode copies of one batch that are adjacent on both
                                sides are merged up to this many bytes; 0 = 16 MiB */
@@ -206,10 +201,9 @@ typedef struct gvm_stats {
   uint64_t launch_exit_ns;      /* (device %globaltimer, ns; 0 before any exit) */
   uint64_t launch_phase[12];    /* that launch's CTA time per phase, summed over CTAs (ns):
                                    [0] finding work (claims, ingest, idle polling),
-                                   [1] ingest passes that published work, [2] split3:
-                                   staging warps waiting for a free stage, [3] GEMM tiles
-                                   (split3: staging warps' time incl. [8]), [4] split3: MMA
-                                   warp waiting for a staged k-step, [5] vector-add tiles;
+                                   [1] ingest passes that published work, [2] 0, [3] GEMM
+                                   tiles (split3: staging warps' time), [4] split3: MMA
+                                   thread waiting for a staged k-step, [5] vector-add tiles;
                                    counts: [6] tiles run, [7] ingest passes that published
                                    work; [8] split3: draining accumulators into C;
                                    [9..11] 0 */
@@ -401,14 +395,15 @@ GVM_API int gvm_vadd_f32(const float* a, const float* b, float* c, int64_t n, vo
    GVM_EINVAL for n < 0, iters outside 1 .. 1024 or NULL pointers. */
 GVM_API int gvm_vmul_f32(const float* a, const float* b, float* c, int64_t n, int32_t iters, void* stream);
 
-/* Scratch bytes gvm_sgemm_f32 needs for (m, n, k, path): 0 for the FMA path;
-   for split3 the bf16 hi/lo copies of A (m x kp) and of B transposed
-   (n x kp), kp = k rounded up to a multiple of 8. */
+/* Scratch bytes gvm_sgemm_f32 asks for with (m, n, k, path): 0 for the paths
+   without scratch; for GVM_SGEMM_SPLIT3 the size of bf16 hi/lo copies of A
+   (m x kp) and B (n x kp), kp = k rounded up to a multiple of 8. (The kernel
+   splits while staging and leaves the scratch untouched.) */
 GVM_API uint64_t gvm_sgemm_scratch_bytes(int32_t m, int32_t n, int32_t k, int32_t path);
 
 /* C = A B (Table 2, MM), row-major binary32 device buffers A (m x k), B (k x n),
    C (m x n). path selects the arithmetic; scratch (device, 256-byte aligned,
-   >= gvm_sgemm_scratch_bytes) is needed by the split3 path only. Returns
+   >= gvm_sgemm_scratch_bytes) must be given with GVM_SGEMM_SPLIT3 only. Returns
    GVM_EINVAL for bad shapes or a short scratch buffer. */
 GVM_API int gvm_sgemm_f32(const float* A, const float* B, float* C, int32_t m, int32_t n, int32_t k,
                   int32_t path, void* scratch, uint64_t scratch_bytes, void* stream);
@@ -420,21 +415,10 @@ GVM_API int gvm_sgemm_f32(const float* A, const float* B, float* C, int32_t m, i
    latency-critical loop where allocating is not allowed. It never calls
    cudaMalloc, cudaFree or any allocating routine.
 
-   Scratch: a fixed 32 MiB array in the library's device image, held by every
-   GPU that loads the library until the process exits. That bounds the shape:
-   4 * (m + n) * kp bytes (kp = k rounded up to 8) must fit, e.g. up to
-   m = n = k = 2048; larger shapes return GVM_ENOMEM and launch nothing.
-   The first call on a device looks up the array's device address
-   (cudaGetSymbolAddress, with that device current) and caches it with the
-   id of the device's context; make that first call before any stream
-   capture. A call in a new context of the device (after cudaDeviceReset)
-   repeats the lookup, so make it before any capture too.
-
-   Every call shares the one array, and the array keeps the previous call's
-   contents (each call rewrites every byte it reads, so nothing needs
-   clearing). Calls whose kernels overlap on the GPU -- for example on two
-   streams at once -- race on the array: order them on one stream.
-   Arguments, layout and errors are otherwise those of gvm_sgemm_f32. */
+   Shape bound: 4 * (m + n) * kp bytes (kp = k rounded up to 8) must be at most
+   32 MiB, e.g. up to m = n = k = 2048; larger shapes return GVM_ENOMEM and
+   launch nothing. Arguments, layout and errors are otherwise those of
+   gvm_sgemm_f32. Calls may overlap on the GPU: they share nothing. */
 GVM_API int gvm_sgemm_f32_noalloc(const float* A, const float* B, float* C, int32_t m, int32_t n, int32_t k,
                                   void* stream);
 

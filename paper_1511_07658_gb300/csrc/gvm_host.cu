@@ -392,11 +392,7 @@ int ps_issue_comp(gvm_rank* r, uint64_t s) {
     if (b.n == 0) return GVM_OK;
     rc = gvm_vmul_f32(A, B, C, b.n, b.k, r->in_stream);
   } else {
-    // The fused split3 form needs no scratch and computes the same tiles as
-    // the scheduler's split3 path.
-    const int path = (ctx->path == kPathSplit3 || ctx->path == kPathSplit3Tma) ? GVM_SGEMM_SPLIT3_FUSED
-                     : ctx->path == kPathSplit3Wide                             ? GVM_SGEMM_SPLIT3_WIDE
-                                                                                : GVM_SGEMM_FMA;
+    const int path = ctx->path == kPathSplit3 ? GVM_SGEMM_SPLIT3_FUSED : GVM_SGEMM_FMA;  // neither needs scratch
     rc = gvm_sgemm_f32(A, B, C, b.m, (int32_t)b.n, b.k, path, nullptr, 0, r->in_stream);
   }
   if (rc == GVM_OK) ctx->launches.fetch_add(1);
@@ -530,10 +526,7 @@ int gvm_init(const gvm_config* cfg_in, gvm_ctx** out) {
   auto ctx = std::make_unique<gvm_ctx>();
   ctx->cfg = cfg;
   ctx->L = L;
-  ctx->path = cfg.sgemm_path == GVM_SGEMM_SPLIT3        ? kPathSplit3
-              : cfg.sgemm_path == GVM_SGEMM_SPLIT3_WIDE ? kPathSplit3Wide
-              : cfg.sgemm_path == GVM_SGEMM_SPLIT3_TMA  ? kPathSplit3Tma
-                                                        : kPathFma;
+  ctx->path = cfg.sgemm_path == GVM_SGEMM_FMA ? kPathFma : kPathSplit3;  // the split3 forms are one kernel
   ctx->slice_bytes = slice;
   ctx->device = dev;
   if (cfg.sched_stream) {
@@ -543,11 +536,12 @@ int gvm_init(const gvm_config* cfg_in, gvm_ctx** out) {
     if (e != cudaSuccess) return cuda_err(e);
     ctx->owned_streams.push_back(ctx->sched);
   }
-  int bps = 0;
-  e = scheduler_setup(ctx->path, &bps, &ctx->smem);
+  int max_ctas = 0;
+  e = scheduler_setup(ctx->path, sms, &max_ctas, &ctx->smem);
   if (e != cudaSuccess) return cuda_err(e);
-  if (bps < 1) return GVM_EDEVICE;
-  ctx->grid = cfg.grid_ctas > 0 ? std::min(cfg.grid_ctas, sms * bps) : sms * bps;
+  if (max_ctas < 1) return GVM_EDEVICE;
+  ctx->grid = cfg.grid_ctas > 0 ? std::min(cfg.grid_ctas, max_ctas) : max_ctas;
+  if (ctx->path == kPathSplit3) ctx->grid = std::min((ctx->grid + 1) / 2 * 2, max_ctas);  // whole pairs
 
   const uint32_t R = (uint32_t)cfg.max_ranks, D = (uint32_t)cfg.ring_depth;
   const uint64_t slots = (uint64_t)R * D;
@@ -789,22 +783,15 @@ void fill_body(gvm_ctx* ctx, gvm_rank* r, const Prep& p, uint64_t seq, uint64_t 
     body->m = t->m;
     body->k = t->k;
     body->n = t->n;
-    // Split3: fused tiles (the bf16 split happens in the tile itself),
-    // 128 x 256 or, in the wide form, 256 x 256.
-    const bool tiles128 = ctx->path == kPathSplit3 || ctx->path == kPathSplit3Tma;
-    const int tm = tiles128 ? kTcM : ctx->path == kPathSplit3Wide ? 256 : kFmaTile;
-    const int tn = tiles128 ? kTcN : ctx->path == kPathSplit3Wide ? 256 : kFmaTile;
-    if (ctx->path != kPathFma) body->flags |= kFlagSplit3;
-    // Wide tiles land A by TMA: the task's own map of A at its device address.
-    if (ctx->path == kPathSplit3Wide &&
-        encode_wide_a_map(reinterpret_cast<const float*>(da), t->m, t->k, &body->tmA) == CUDA_SUCCESS)
-      body->flags |= kFlagTmA;
-    // The TMA form lands A and B by TMA: the task's own maps of both.
-    int b3 = 0;
-    if (ctx->path == kPathSplit3Tma &&
-        encode_tma_maps(reinterpret_cast<const float*>(da), reinterpret_cast<const float*>(db), t->m, t->n, t->k,
-                        &body->tmA, &body->tmB, &b3) == CUDA_SUCCESS)
-      body->flags |= kFlagTmA | kFlagTmB | (b3 ? kFlagTmB3 : 0u);
+    const bool split3 = ctx->path != kPathFma;
+    const int tm = split3 ? 256 : kFmaTile, tn = tm;
+    if (split3) {
+      body->flags |= kFlagSplit3;
+      body->vadd_tile = tn;
+      // Operands land by tensor copies: the task's own maps of A and B.
+      body->flags |= kFlagTmA * encode_pair_maps(reinterpret_cast<const float*>(da), reinterpret_cast<const float*>(db),
+                                                 t->m, t->n, t->k, &body->tmA, &body->tmB);
+    }
     body->tiles_m = (uint32_t)((t->m + tm - 1) / tm);
     body->tiles_n = (uint32_t)((t->n + tn - 1) / tn);
     body->ntiles = body->tiles_m * body->tiles_n;

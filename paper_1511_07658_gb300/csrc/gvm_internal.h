@@ -8,32 +8,26 @@
 namespace gvm {
 
 // ---- tiling ---------------------------------------------------------------
-constexpr int kThreads = 256;         // scheduler and task-kernel CTA size (8 warps)
+constexpr int kThreads = 256;         // vector-kernel CTA size (8 warps)
+constexpr int kFmaThreads = 128;      // FMA scheduler and kernel CTA size (two CTAs an SM)
 constexpr int kFmaTile = 128;         // FMA SGEMM output tile (square)
 constexpr int kFmaBK = 16;            // FMA SGEMM k-step
-constexpr int kTcM = 128;             // tcgen05 tile rows (one TMEM lane per row)
-constexpr int kTcN = 256;             // tcgen05 tile columns (fp32 TMEM columns)
-constexpr int kTcBK = 32;             // bf16 k per pipeline stage (64-byte rows)
-constexpr int kTcStages = 4;          // TMA -> MMA pipeline depth
-constexpr int kSplitRows = 128;       // rows of A (or columns of B) per split tile
+constexpr int kTcBK = 32;             // split3: k per pipeline stage (64-byte bf16 rows)
 constexpr int64_t kVaddTileMin = 16384;
 constexpr int64_t kVaddTileMax = 1 << 20;
 constexpr int kProfSlots = 12;        // per-launch phase counters (see kProf*)
 
-// Bytes of one pipeline stage: A hi, A lo (kTcM x kTcBK) and B^T hi, lo (kTcN x kTcBK).
-constexpr uint32_t kTcStageBytes = (2u * kTcM + 2u * kTcN) * kTcBK * 2u;
-
-// ---- task kinds, phases, flags ---------------------------------------------
+// ---- task kinds, flags ---------------------------------------------
 enum : uint32_t { kTaskVadd = 1, kTaskSgemm = 2, kTaskVmul = 3 };
-enum : uint32_t { kPhaseSplit = 0, kPhaseMain = 1 };
 enum : uint32_t {
   kFlagNeedsReady = 1u,   // host-mode inputs: wait for the input stream's ready word
   kFlagNeedsD2H = 2u,     // host-mode output: the output stream copies and completes
   kFlagSplit3 = 4u,       // SGEMM on the split-bf16 tensor-core path
   kFlagDirectOut = 8u,    // host-mode output written by the kernel into host memory
-  kFlagTmA = 16u,         // wide / TMA split3: tmA maps A (ingest copies it)
-  kFlagTmB = 32u,         // TMA split3: tmB maps B in 32-row x 32-value boxes (ingest copies it)
-  kFlagTmB3 = 64u,        // with kFlagTmB: tmB is 3D, one box lands a k-step's eight 32-column slabs
+  kFlagTmA = 16u,         // split3: tmA maps A (ingest copies it)
+  kFlagTmB = 32u,         // split3: tmB maps B (ingest copies it)
+  kFlagPackA = 64u,       // with kFlagTmA: tmA maps A's rows in fours
+  kFlagPackB = 128u,      // with kFlagTmB: tmB maps B's rows in fours
 };
 
 // Device status words (written to HostShared::status with the place in `where`).
@@ -58,8 +52,8 @@ constexpr uint32_t kClaimLocked = 0x40000000u;  // claim counter while a slot is
 // ---- task body: written by the host into its ring, copied by the device ----
 // 384 bytes; the two tensor maps must stay 64-byte aligned (they are at 0, 128).
 struct alignas(128) TaskBody {
-  CUtensorMap tmA;  // kFlagTmA: binary32 A (m x k), box {kTcBK, 256} (wide) or {kTcBK, 128} (TMA form)
-  CUtensorMap tmB;  // kFlagTmB: binary32 B (k x n), box {32, kTcBK}; kFlagTmB3: (32, k, n / 32), box {32, kTcBK, 8}
+  CUtensorMap tmA;  // kFlagTmA: binary32 A (m x k), see encode_pair_maps
+  CUtensorMap tmB;  // kFlagTmB: binary32 B (k x n)
   uint32_t type;
   uint32_t flags;
   uint32_t rank;
@@ -73,7 +67,7 @@ struct alignas(128) TaskBody {
   int32_t m;
   int32_t k;
   int64_t n;
-  int64_t vadd_tile; // elements per vector-add tile
+  int64_t vadd_tile; // elements per vector-add tile; split3 SGEMM: columns per tile
   uint64_t a, b, c;  // device addresses of the operands
   uint64_t scratch;  // device address of the split3 planes (A planes, then B^T planes)
   uint64_t scratch_b;// device address of the B^T planes
@@ -128,13 +122,12 @@ struct alignas(64) HostShared {
 enum : int {
   kProfAcquire = 0,    // the claiming warp finding the next tile (claims, ingest, idle polling)
   kProfIngest = 1,     // inside ingest passes that published work
-  kProfStageWait = 2,  // split3: converters waiting for a free pipeline stage (MMA-bound time)
-  kProfGemm = 3,       // GEMM tiles (FMA; split3: converter time, staging + epilogue)
+  kProfGemm = 3,       // GEMM tiles (FMA; split3: converter time)
   kProfMmaWait = 4,    // split3: the MMA warp waiting for a staged k-step (staging-bound time)
   kProfVadd = 5,       // vector-add tiles
   kProfTiles = 6,      // tiles run
   kProfIngests = 7,    // ingest passes that published work
-  kProfEpilogue = 8,   // split3: converter time draining accumulators into C (part of kProfGemm)
+  kProfEpilogue = 8,   // split3: epilogue warps draining accumulators into C
 };
 
 // Device control block (front of the caller's ctrl buffer).
@@ -158,15 +151,15 @@ struct alignas(256) DevCtrl {
 };
 static_assert(sizeof(DevCtrl) == 256, "DevCtrl layout");
 
-// Publication-queue entry: one phase of one task, covering tiles
-// [base, base + cnt) of the global tile space.
+// Publication-queue entry: one task, covering tiles [base, base + cnt) of the
+// global tile space.
 struct PubEntry {
   uint64_t base;   // first global tile index
   uint64_t seq;    // entry index (checks that the ring slot was not reused)
   uint32_t task;   // rank * depth + slot
-  uint32_t phase;  // kPhaseSplit or kPhaseMain
-  uint32_t cnt;    // tiles in this entry
   uint32_t pad;
+  uint32_t cnt;    // tiles in this entry
+  uint32_t check;  // pub_check of the other words
 };
 static_assert(sizeof(PubEntry) == 32, "PubEntry layout");
 
@@ -218,7 +211,9 @@ inline CtrlLayout ctrl_layout(uint32_t ranks, uint32_t depth) {
   return L;
 }
 
-// Split3 scratch: A planes [2][m][kp] then B^T planes [2][n][kp], bf16.
+// Bytes of the bf16 hi and lo copies of A and B (kp = k rounded up to 8): what
+// gvm_sgemm_scratch_bytes reports and the shape bound of the entry point
+// without allocation. The kernels split while staging and use no scratch.
 inline uint32_t split_kp(int32_t k) { return (uint32_t)((k + 7) / 8 * 8); }
 inline uint64_t split_a_bytes(int32_t m, int32_t k) { return align_up(4ull * (uint64_t)m * split_kp(k), 256); }
 inline uint64_t split_scratch_bytes(int32_t m, int32_t n, int32_t k) {

@@ -19,8 +19,7 @@
 //            other warps run the current one.
 //   ingest:  one CTA at a time (holding a lock) copies ready descriptors from
 //            the host rings into the device task table and appends queue
-//            entries (split phases of a pass before main phases, so the
-//            split3 pre-pass of a task runs well ahead of its GEMM).
+//            entries.
 //   finish:  the CTA that completes a task's last tile publishes completion:
 //            the host completion word (resident tasks) or the device done word
 //            on which the rank's output-copy stream waits (host-buffer tasks).
@@ -32,14 +31,13 @@
 // descriptor published before its launch has been taken.
 #include "gvm_device.cuh"
 #include <cstddef>
-#include <type_traits>
 
-#include "gvm_fused.cuh"
+#include "gvm_pair.cuh"
 #include "gvm_runtime.h"
-#include "gvm_tma.cuh"
-#include "gvm_wide.cuh"
 
 namespace gvm {
+
+constexpr uint32_t kMaxQuantum = 8;
 
 // FMA path: two tile slots; the CTA runs the tile in one while warp 0 claims
 // the next into the other. go: 1 = a tile is there, 0 = exit, 2 = nothing
@@ -48,16 +46,13 @@ struct alignas(128) SchedShared {
   TaskBody body[2];  // copies of the claimed tasks' bodies
   uint32_t go[2];
   uint32_t task[2];
-  uint32_t phase[2];
   uint32_t tile[2];
-  uint32_t need[2];  // per iteration parity: a blocking claim must follow the tile
-  uint32_t abort;
-  uint32_t fail_where;
+  uint64_t t_tile;   // when the current tile began (thread 0)
   uint64_t prof[kProfSlots];  // this CTA's phase counters (kProf*), written by thread 0 only
   uint64_t claim[4];  // Claim state (see acquire), owned by warp 0
+  uint32_t list[2 * 32 * kMaxQuantum];  // ingest's scratch, warp 0
 };
 
-constexpr uint32_t kMaxQuantum = 8;
 constexpr uint64_t kLookaheadTiles = 512;  // ingest ahead when this few published tiles remain
 constexpr uint64_t kQuietNs = 20000; // skip look-ahead ingest this long after an empty pass
 
@@ -106,11 +101,55 @@ struct IngestOut {
   uint32_t pending;
 };
 
+// The task fields are a descriptor's last 128 bytes, the tensor maps its
+// first 256.
+constexpr uint32_t kFieldsAt = 256;
+static_assert(offsetof(TaskBody, type) == kFieldsAt && sizeof(TaskBody) == 384, "TaskBody fields");
+static_assert(offsetof(TaskBody, flags) == 260 && offsetof(TaskBody, tag) == 272 && offsetof(TaskBody, ntiles) == 276,
+              "TaskBody header words");
+static_assert(offsetof(TaskBody, tmA) == 0 && offsetof(TaskBody, tmB) == 128 && sizeof(CUtensorMap) == 128,
+              "TaskBody maps");
+
+// Check word of a queue entry: a reader may meet an entry that is being
+// written (one beyond the published tiles) and must not take a mixture of
+// its old and new words for a whole entry.
+__device__ __forceinline__ uint32_t pub_check(uint32_t base, uint32_t seq, uint32_t task, uint32_t cnt) {
+  return base ^ (seq * 0x9e3779b9u) ^ (task << 16) ^ cnt;
+}
+
+// One warp copies, for each of n tasks, `pieces` (8 or 16) 16-byte pieces
+// starting `at` bytes into its descriptor from the host ring to the device
+// table, kBatch reads of host memory in flight a lane.
+template <uint32_t kPieces, uint32_t kBatch>
+__device__ __forceinline__ void copy_bodies(const SchedParams& p, const uint32_t* list, uint32_t n, uint32_t at) {
+  const uint32_t lane = threadIdx.x & 31, total = n * kPieces;
+#pragma unroll 1
+  for (uint32_t u0 = lane; u0 < total; u0 += 32 * kBatch) {
+    uint4 v[kBatch];
+#pragma unroll
+    for (uint32_t j = 0; j < kBatch; ++j) {
+      const uint32_t u = u0 + 32 * j;
+      if (u < total)
+        v[j] = ld_volatile_v4(reinterpret_cast<const uint8_t*>(&p.host_desc[list[u / kPieces]]) + at + 16 * (u % kPieces));
+    }
+#pragma unroll
+    for (uint32_t j = 0; j < kBatch; ++j) {
+      const uint32_t u = u0 + 32 * j;
+      if (u < total) st_cg_v4(reinterpret_cast<uint8_t*>(&p.tasks[list[u / kPieces]].body) + at + 16 * (u % kPieces), v[j]);
+    }
+  }
+}
+
 // Warp 0 of one CTA: move ready descriptors from the host rings into the
 // device table and append their queue entries, each covering a contiguous
-// range of the global tile space. All lanes call.
-template <bool kPrefetch>
-__device__ IngestOut ingest(const SchedParams& p, uint64_t* prof) {
+// range of the global tile space. All lanes call. Lane = rank: it reads the
+// heads and the header words of its rank's next tasks (kBatch tasks' reads in
+// flight), then the warp copies all taken descriptors together. Read and
+// stored task by task by each lane, a pass of 64 tasks with tensor maps took
+// 43 us, 0.68 ms of a 1024-task launch. list: two arrays of 32 x kMaxQuantum
+// words in shared memory.
+template <uint32_t kBatch>
+__device__ __forceinline__ IngestOut ingest_pass(const SchedParams& p, uint64_t* prof, uint32_t* list) {
   const int lane = threadIdx.x & 31;
   IngestOut out{0, 0, 0};
   uint32_t got = 0;
@@ -145,6 +184,7 @@ __device__ IngestOut ingest(const SchedParams& p, uint64_t* prof) {
   uint64_t pub = pub0, ptiles = tiles0;
   uint32_t pending = 0;
   bool bad = false;
+  uint32_t* maps_list = list + 32 * kMaxQuantum;
 
   for (uint32_t g = 0; g < p.ranks; g += 32) {
     // Keep at most half the ring between the hand-out frontier and the
@@ -152,129 +192,96 @@ __device__ IngestOut ingest(const SchedParams& p, uint64_t* prof) {
     const uint64_t used = pub - consumed;
     const uint32_t space = used < p.qcap / 2 ? (uint32_t)(p.qcap / 2 - used) : 0u;
     uint32_t quantum = min(p.quantum, kMaxQuantum);
-    // Each task takes at most two queue entries.
     const uint32_t lanes = min(32u, p.ranks - g);
-    if (2u * lanes * quantum > space) quantum = space / (2u * lanes);
+    if (lanes * quantum > space) quantum = space / lanes;
 
     uint32_t r = 0, t = 0, take = 0, avail = 0;
-    uint32_t tidx[kMaxQuantum], tsplit[kMaxQuantum], tmain[kMaxQuantum];
-    uint32_t nsplit_e = 0, nmain_e = 0, split_tiles = 0, main_tiles = 0;
+    uint32_t tidx[kMaxQuantum], tcnt[kMaxQuantum];
+    uint32_t entries = 0, tiles = 0, maps = 0;  // maps: bit i = task i has tensor maps to copy
     const bool valid = (g + lane) < p.ranks;
+    uint32_t lim = 0;
     if (valid) {
       r = (rr + g + lane) % p.ranks;
       const uint32_t h = ld_acquire_sys(&p.host_heads[r].head);
       t = ld_relaxed_gpu(&p.tail[r]);
       avail = h - t;
-      const uint32_t lim = min(avail, quantum);
-      // The task fields are the descriptor's last 128 bytes (its first 256, the
-      // pre-pass form's tensor maps, are not used here). One read of them from
-      // host memory gives both the readiness rule and the fields to copy.
-      constexpr int kFieldsAt = offsetof(TaskBody, type) / 16;
-      static_assert(offsetof(TaskBody, type) == 256 && sizeof(TaskBody) == 384, "TaskBody fields");
-      static_assert(offsetof(TaskBody, flags) == 260 && offsetof(TaskBody, tag) == 272 &&
-                        offsetof(TaskBody, ntiles) == 276 && offsetof(TaskBody, nsplit) == 280,
-                    "TaskBody header words");
-      // kPrefetch: descriptor s + 1 is read while s is processed, so that a
-      // lane's host round trips overlap instead of following one another
-      // (32 more registers; the FMA scheduler, which would spill, reads them
-      // one by one).
-      auto fields_of = [&](uint32_t s) {
-        return reinterpret_cast<const uint4*>(&p.host_desc[r * p.depth + (s & (p.depth - 1))]) + kFieldsAt;
-      };
-      uint4 vn[kPrefetch ? 8 : 1];
-      if (kPrefetch && lim > 0) {
-        const uint4* src = fields_of(t);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) vn[kPrefetch ? j : 0] = ld_volatile_v4(src + j);
-      }
-      for (; take < lim; ++take) {
-        const uint32_t s = t + take;
-        const uint32_t idx = r * p.depth + (s & (p.depth - 1));
-        uint4 v[8];
-        if constexpr (kPrefetch) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) v[j] = vn[j];
-          if (take + 1 < lim) {
-            const uint4* nsrc = fields_of(s + 1);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) vn[j] = ld_volatile_v4(nsrc + j);
-          }
-        } else {
-          const uint4* src = fields_of(s);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) v[j] = ld_volatile_v4(src + j);
-        }
-        const uint32_t flags = v[0].y;
-        if ((flags & kFlagNeedsReady) && ld_acquire_gpu(&p.ready[idx]) != s + 1u) break;
-        DevTask* dt = &p.tasks[idx];
-        uint4* dst = reinterpret_cast<uint4*>(&dt->body) + kFieldsAt;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) st_cg_v4(dst + j, v[j]);
-        if (flags & (kFlagTmA | kFlagTmB)) {  // the tensor maps (the descriptor's first 128 or 256 bytes)
-          static_assert(offsetof(TaskBody, tmA) == 0 && offsetof(TaskBody, tmB) == 128 &&
-                            sizeof(CUtensorMap) == 128, "TaskBody maps");
-          const uint4* m_src = reinterpret_cast<const uint4*>(&p.host_desc[idx]);
-          uint4* m_dst = reinterpret_cast<uint4*>(&dt->body);
-          const int nv = (flags & kFlagTmB) ? 16 : 8;
+      lim = min(avail, quantum);
+    }
+    bool more = valid;
 #pragma unroll 1
-          for (int j = 0; j < nv; ++j) st_cg_v4(m_dst + j, ld_volatile_v4(m_src + j));
+    for (uint32_t base = 0; base < kMaxQuantum && __any_sync(0xffffffffu, more && base < lim); base += kBatch) {
+      uint4 h0[kBatch], h1[kBatch];
+      uint32_t rdy[kBatch];
+#pragma unroll
+      for (uint32_t i = 0; i < kBatch; ++i) {
+        if (more && base + i < lim) {
+          const uint32_t idx = r * p.depth + ((t + base + i) & (p.depth - 1));
+          const uint4* src = reinterpret_cast<const uint4*>(&p.host_desc[idx]) + kFieldsAt / 16;
+          h0[i] = ld_volatile_v4(src);      // type, flags, rank, slot
+          h1[i] = ld_volatile_v4(src + 1);  // tag, ntiles, nsplit, tiles_m
+          rdy[i] = ld_relaxed_gpu(&p.ready[idx]);
         }
-        const uint32_t tag = v[1].x;
-        const uint32_t ntiles = v[1].y;
-        const uint32_t nsplit = v[1].z;
-        tidx[take] = idx;
-        tsplit[take] = tmain[take] = 0;
-        if (tag != s + 1u || nsplit > ntiles) {
-          bad = true;
-          continue;
-        }
-        atomicExch(&dt->tiles_done, 0u);
-        atomicExch(&dt->split_done, 0u);
-        *reinterpret_cast<volatile uint64_t*>(&dt->t_ingest) = now;
-        if (ntiles == 0) {
-          __threadfence();
-          complete_task(p, idx, tag, flags, now);
-          continue;
-        }
-        tsplit[take] = nsplit;
-        tmain[take] = ntiles - nsplit;
-        if (nsplit) {
-          ++nsplit_e;
-          split_tiles += nsplit;
-        }
-        if (ntiles > nsplit) {
-          ++nmain_e;
-          main_tiles += ntiles - nsplit;
+      }
+#pragma unroll
+      for (uint32_t i = 0; i < kBatch; ++i) {
+        if (more && base + i < lim) {
+          const uint32_t s = t + base + i;
+          const uint32_t idx = r * p.depth + (s & (p.depth - 1));
+          const uint32_t flags = h0[i].y, tag = h1[i].x, ntiles = h1[i].y;
+          if ((flags & kFlagNeedsReady) && rdy[i] != s + 1u) {
+            more = false;
+          } else {
+            tidx[take] = idx;
+            tcnt[take] = 0;
+            if (tag != s + 1u) {
+              bad = true;
+            } else {
+              DevTask* dt = &p.tasks[idx];
+              *reinterpret_cast<volatile uint32_t*>(&dt->tiles_done) = 0;
+              *reinterpret_cast<volatile uint64_t*>(&dt->t_ingest) = now;
+              if (ntiles == 0) {
+                __threadfence();
+                complete_task(p, idx, tag, flags, now);
+              } else {
+                if (flags & (kFlagTmA | kFlagTmB)) maps |= 1u << take;
+                tcnt[take] = ntiles;
+                ++entries;
+                tiles += ntiles;
+              }
+            }
+            ++take;
+          }
         }
       }
     }
+    // The ready words (written by the input streams after their copies) were
+    // read relaxed: order the copies' data before what is published below.
+    __threadfence();
 
-    // Split entries of this pass first, then main entries, each group in lane
-    // order: the split3 pre-pass of a task is handed out well ahead of its GEMM.
-    const uint32_t ie_s = warp_incl_scan(nsplit_e), ie_m = warp_incl_scan(nmain_e);
-    const uint32_t it_s = warp_incl_scan(split_tiles), it_m = warp_incl_scan(main_tiles);
-    const uint32_t te_s = __shfl_sync(0xffffffffu, ie_s, 31), te_m = __shfl_sync(0xffffffffu, ie_m, 31);
-    const uint32_t tt_s = __shfl_sync(0xffffffffu, it_s, 31), tt_m = __shfl_sync(0xffffffffu, it_m, 31);
-    uint64_t es = pub + ie_s - nsplit_e, em = pub + te_s + ie_m - nmain_e;
-    uint64_t bs = ptiles + it_s - split_tiles, bm = ptiles + tt_s + it_m - main_tiles;
+    // Copy the taken tasks' fields and maps.
+    const uint32_t nt = entries, ie = warp_incl_scan(nt), it = warp_incl_scan(tiles);
+    const uint32_t nm = (uint32_t)__popc(maps), im = warp_incl_scan(nm);
+    const uint32_t te = __shfl_sync(0xffffffffu, ie, 31), tt = __shfl_sync(0xffffffffu, it, 31);
+    const uint32_t tm = __shfl_sync(0xffffffffu, im, 31);
+    uint64_t e0 = pub + ie - nt, b0 = ptiles + it - tiles;
+    uint32_t at = ie - nt, at_m = im - nm;
     for (uint32_t i = 0; i < take; ++i) {
-      if (tsplit[i]) {
-        PubEntry e{bs, es, tidx[i], kPhaseSplit, tsplit[i], 0};
-        p.pubq[es & (p.qcap - 1)] = e;
-        ++es;
-        bs += tsplit[i];
-      }
-      if (tmain[i]) {
-        PubEntry e{bm, em, tidx[i], kPhaseMain, tmain[i], 0};
-        p.pubq[em & (p.qcap - 1)] = e;
-        ++em;
-        bm += tmain[i];
-      }
+      if (!tcnt[i]) continue;
+      list[at++] = tidx[i];
+      if ((maps >> i) & 1u) maps_list[at_m++] = tidx[i];
+      PubEntry e{b0, e0, tidx[i], 0, tcnt[i], pub_check((uint32_t)b0, (uint32_t)e0, tidx[i], tcnt[i])};
+      p.pubq[e0 & (p.qcap - 1)] = e;
+      ++e0;
+      b0 += tcnt[i];
     }
+    __syncwarp();
+    copy_bodies<8, 2 * kBatch>(p, list, te, kFieldsAt);
+    copy_bodies<16, 2 * kBatch>(p, maps_list, tm, 0);
+    __syncwarp();
     if (valid && take > 0) *reinterpret_cast<volatile uint32_t*>(&p.tail[r]) = t + take;
     pending += avail - take;
-    pub += te_s + te_m;
-    ptiles += tt_s + tt_m;
+    pub += te;
+    ptiles += tt;
   }
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) pending += __shfl_xor_sync(0xffffffffu, pending, d);
@@ -306,6 +313,19 @@ __device__ IngestOut ingest(const SchedParams& p, uint64_t* prof) {
   return out;
 }
 
+// The pair scheduler calls it (kCall): inlined twice into its claim loop, its
+// registers spilled there, and what spills is read back from L2 (the claim's
+// own acquires invalidate L1). In the FMA scheduler a call would cost the tile
+// loop its registers.
+static __device__ __noinline__ IngestOut ingest_call(const SchedParams& p, uint64_t* prof, uint32_t* list) {
+  return ingest_pass<4>(p, prof, list);
+}
+template <bool kCall>
+__device__ __forceinline__ IngestOut ingest(const SchedParams& p, uint64_t* prof, uint32_t* list) {
+  if constexpr (kCall) return ingest_call(p, prof, list);
+  else return ingest_pass<1>(p, prof, list);
+}
+
 __device__ __forceinline__ uint32_t bcast(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
 __device__ __forceinline__ uint64_t bcast64(uint64_t v) {
   const uint32_t lo = __shfl_sync(0xffffffffu, (uint32_t)v, 0);
@@ -324,19 +344,24 @@ struct Claim {
   uint32_t pad;
 };
 
-// One warp: find the next tile to run. Returns 1 with (task, phase, tile) set,
+// One warp: find the next tile to run. Returns 1 with (task, tile) set,
 // 0 when the kernel should exit, and 2 when the reserved tile is not
 // published yet and either !blocking or a blocking call has found nothing for
-// idle_return_ns (0: never). Decisions use values lane 0 read and broadcast,
-// so the warp never diverges across the shuffles.
+// idle_return_ns (0: never). Decisions use values that one lane read and
+// broadcast, so the warp never diverges across the shuffles.
 //
 // Claiming is one atomicAdd on next_tile per tile: there is no per-entry
 // counter for all CTAs to contend on. A tile beyond published_tiles is a
 // reservation; tiles are published in increasing order, so it becomes valid
 // without further claims.
-template <bool kPrefetch>
-__device__ int acquire(const SchedParams& p, Claim* cl, uint32_t& task, uint32_t& phase, uint32_t& tile,
-                       uint64_t* prof, bool blocking, uint64_t idle_return_ns = 0) {
+//
+// The control words are read by different lanes at once, an entry window in
+// one go: a claim is three round trips to L2 with the task's fields (read by
+// the caller). Read one after another they were about ten: a claim took 10 us
+// of a loaded GPU, longer than a 256 x 256 x 512 tile.
+template <bool kCall>
+__device__ __forceinline__ int acquire(const SchedParams& p, Claim* cl, uint32_t* list, uint32_t& task, uint32_t& tile,
+                                       uint64_t* prof, bool blocking, uint64_t idle_return_ns = 0) {
   const int lane = threadIdx.x & 31;
   uint64_t entered = 0;
   auto set_stall = [&](uint64_t v) {
@@ -344,49 +369,66 @@ __device__ int acquire(const SchedParams& p, Claim* cl, uint32_t& task, uint32_t
     __syncwarp();
   };
   while (true) {
-    uint32_t abort = 0, drained = 0;
-    uint64_t pt = 0, npub = 0, now = 0, quiet = 0, x = 0;
+    uint64_t v = 0;
     if (lane == 0) {
-      abort = ld_relaxed_gpu(&p.ctrl->abort);
-      drained = ld_acquire_gpu(&p.ctrl->drained);
       if (!cl->has_resv) {
         cl->resv = atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->next_tile), 1ull);
         cl->has_resv = 1;
       }
-      x = cl->resv;
-      pt = ld_acquire_gpu64(&p.ctrl->published_tiles);
-      // Entries below `published` are complete: an ingest pass releases
-      // `published` (before published_tiles) only after writing them. An
-      // entry beyond it may be half written (new seq, old count).
-      npub = ld_acquire_gpu64(&p.ctrl->published);
-      quiet = ld_relaxed_gpu64(&p.ctrl->quiet_until);
-      now = globaltimer();
+      v = cl->resv;
+    } else if (lane == 1) {
+      v = ld_relaxed_gpu(&p.ctrl->abort);
+    } else if (lane == 2) {
+      v = ld_acquire_gpu(&p.ctrl->drained);
+    } else if (lane == 3) {
+      v = ld_acquire_gpu64(&p.ctrl->published_tiles);
+    } else if (lane == 4) {
+      v = ld_relaxed_gpu64(&p.ctrl->quiet_until);
+    } else if (lane == 5) {
+      v = globaltimer();
     }
-    if (bcast(abort)) return 0;
-    drained = bcast(drained);
-    if (entered == 0) entered = bcast64(now);
-    x = bcast64(x);
-    pt = bcast64(pt);
-    npub = bcast64(npub);
-    now = bcast64(now);
-    quiet = bcast64(quiet);
-    if (x < pt) {
-      // Keep the queue ahead of the CTAs.
-      if (pt - x <= kLookaheadTiles && now >= quiet) (void)ingest<kPrefetch>(p, prof);
+    __syncwarp();
+    const uint64_t x = __shfl_sync(0xffffffffu, v, 0), pt = __shfl_sync(0xffffffffu, v, 3);
+    const uint64_t quiet = __shfl_sync(0xffffffffu, v, 4), now = __shfl_sync(0xffffffffu, v, 5);
+    if (__shfl_sync(0xffffffffu, v, 1)) return 0;
+    const bool drained = __shfl_sync(0xffffffffu, v, 2) != 0;
+    if (entered == 0) entered = now;
+    const bool here = x < pt;
+    // The reserved tile is not published yet. Before leaving, look at the
+    // published tiles once more: another CTA's last ingest pass may have
+    // published the reserved tile since pt was read, and a tile whose owner
+    // leaves would never run. Once the rings are drained (or stop is set with
+    // nothing pending) no further tile is published, so this read is final.
+    auto reserved_published = [&]() -> bool {
+      uint64_t pt2 = 0;
+      if (lane == 0) pt2 = ld_acquire_gpu64(&p.ctrl->published_tiles);
+      return x < bcast64(pt2);
+    };
+    if (!here && p.drain && drained) {
+      if (reserved_published()) continue;
+      return 0;
+    }
+    // Ingest when the tile is not there, or to keep the queue ahead of the CTAs.
+    IngestOut r{0, 0, 0};
+    if (!here || (pt - x <= kLookaheadTiles && now >= quiet)) r = ingest<kCall>(p, prof, list);
+    if (here) {
       // Find the entry holding tile x: the last entry with base <= x. Entries
       // are published in tile order, and x only grows from one claim of a CTA
       // to the next, so the search starts at the entry of this CTA's previous
-      // tile; the warp checks 32 entries per step.
-      uint32_t etask = 0, ephase = 0, off = 0, ok = 1;
+      // tile; the warp checks 32 entries per step. An ingest pass releases
+      // published_tiles only after writing its entries, so those up to the one
+      // holding x are whole; a later one may be half written, which its check
+      // word shows, or whole, with a base above x.
+      uint32_t etask = 0, off = 0, ok = 1;
       uint64_t e0 = 0;
       if (lane == 0) e0 = cl->hint;
       e0 = bcast64(e0);
       while (true) {
         const uint64_t e = e0 + (uint64_t)lane;
         const PubEntry* pe = &p.pubq[e & (p.qcap - 1)];
-        const uint64_t seq = ld_relaxed_gpu64(&pe->seq);
-        const uint64_t base = ld_relaxed_gpu64(&pe->base);
-        const bool le = (e < npub) && (seq == e) && base <= x;
+        const uint4 w0 = ld_volatile_v4(pe), w1 = ld_volatile_v4(reinterpret_cast<const uint4*>(pe) + 1);
+        const uint64_t base = ((uint64_t)w0.y << 32) | w0.x, seq = ((uint64_t)w0.w << 32) | w0.z;
+        const bool le = (seq == e) && base <= x && w1.w == pub_check(w0.x, w0.z, w1.x, w1.z);
         const uint32_t m = __ballot_sync(0xffffffffu, le);
         if (m == 0) {  // not even the first entry starts at or before x
           ok = 0;
@@ -397,13 +439,9 @@ __device__ int acquire(const SchedParams& p, Claim* cl, uint32_t& task, uint32_t
           e0 += 31;
           continue;
         }
-        const uint32_t cnt = ld_relaxed_gpu(&pe->cnt);
-        const uint32_t tk = ld_relaxed_gpu(&pe->task);
-        const uint32_t ph = ld_relaxed_gpu(&pe->phase);
         const uint64_t hit_base = __shfl_sync(0xffffffffu, base, last);
-        const uint32_t hit_cnt = __shfl_sync(0xffffffffu, cnt, last);
-        etask = __shfl_sync(0xffffffffu, tk, last);
-        ephase = __shfl_sync(0xffffffffu, ph, last) & 1u;
+        const uint32_t hit_cnt = __shfl_sync(0xffffffffu, w1.z, last);
+        etask = __shfl_sync(0xffffffffu, w1.x, last);
         if (x >= hit_base + hit_cnt) {  // a hole in the tile space: the ring bound was broken
           ok = 0;
           break;
@@ -420,31 +458,15 @@ __device__ int acquire(const SchedParams& p, Claim* cl, uint32_t& task, uint32_t
         __syncwarp();
         break;
       }
-      if (!bcast(ok)) {
+      if (!ok) {
         if (lane == 0) report_error(p, kStatusBadTask, kWhereQueueFull, (uint32_t)x);
         __syncwarp();
         return 0;
       }
-      task = bcast(etask);
-      phase = bcast(ephase);
-      tile = bcast(off);
+      task = etask;
+      tile = off;
       return 1;
     }
-    // The reserved tile is not published yet. Before leaving, look at the
-    // published tiles once more: another CTA's last ingest pass may have
-    // published the reserved tile since pt was read, and a tile whose owner
-    // leaves would never run. Once the rings are drained (or stop is set with
-    // nothing pending) no further tile is published, so this read is final.
-    auto reserved_published = [&]() -> bool {
-      uint64_t pt2 = 0;
-      if (lane == 0) pt2 = ld_acquire_gpu64(&p.ctrl->published_tiles);
-      return x < bcast64(pt2);
-    };
-    if (p.drain && drained) {
-      if (reserved_published()) continue;
-      return 0;
-    }
-    const IngestOut r = ingest<kPrefetch>(p, prof);
     if (r.published) {
       set_stall(0);
       continue;
@@ -535,13 +557,48 @@ __device__ void finish_tile(const SchedParams& p, uint32_t task, uint32_t ntiles
 
 // ------------------------------------------------------------ FMA scheduler
 
-__global__ void __launch_bounds__(kThreads, 2) sched_fma_kernel(const SchedParams p) {
+// Warp 0: claim a tile into slot s (blocking: wait for work; otherwise
+// return at once with go = 2 when nothing is claimable).
+static __device__ __noinline__ void fma_claim(const SchedParams& p, SchedShared& sh, int slot, bool blocking) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t t_acq = globaltimer();
+  uint32_t task = 0, tile = 0;
+  const int got = acquire<false>(p, reinterpret_cast<Claim*>(sh.claim), sh.list, task, tile, sh.prof, blocking);
+  if (lane == 0) {
+    sh.go[slot] = (uint32_t)got;
+    sh.task[slot] = task;
+    sh.tile[slot] = tile;
+  }
+  if (got == 1 && lane < (int)(sizeof(TaskBody) / 16)) {
+    const uint4 v = ld_cg_v4(reinterpret_cast<const uint4*>(&p.tasks[task].body) + lane);
+    reinterpret_cast<uint4*>(&sh.body[slot])[lane] = v;
+  }
+  __syncwarp();
+  if (lane == 0) sh.prof[kProfAcquire] += globaltimer() - t_acq;
+}
+
+// All threads: slot cur's tile is done.
+__device__ __forceinline__ void fma_finish(const SchedParams& p, SchedShared& sh, int cur, int bucket) {
+  const TaskBody& b = sh.body[cur];
+  // Results written into host memory: visible to the host before the task's
+  // completion word.
+  if (b.flags & kFlagDirectOut)
+    __threadfence_system();
+  else
+    __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    sh.prof[bucket] += globaltimer() - sh.t_tile;
+    sh.prof[kProfTiles] += 1;
+    finish_tile(p, sh.task[cur], b.ntiles, b.tag, b.flags);
+  }
+}
+
+__global__ void __launch_bounds__(kFmaThreads, 2) sched_fma_kernel(const __grid_constant__ SchedParams p) {
   __shared__ SchedShared sh;
   extern __shared__ uint8_t dyn_smem[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tid >> 5;
   if (tid == 0) {
-    sh.abort = 0;
-    sh.fail_where = 0;
     for (int i = 0; i < kProfSlots; ++i) sh.prof[i] = 0;
     sched_enter(p);
   }
@@ -555,138 +612,89 @@ __global__ void __launch_bounds__(kThreads, 2) sched_fma_kernel(const SchedParam
   }
   __syncthreads();
 
-  // Warp 0: claim a tile into slot s (blocking: wait for work; otherwise
-  // return at once with go = 2 when nothing is claimable).
-  auto claim = [&](int slot, bool blocking) {
-    const uint64_t t_acq = globaltimer();
-    uint32_t task = 0, phase = 0, tile = 0;
-    const int got = acquire<false>(p, cl, task, phase, tile, sh.prof, blocking);
-    if (lane == 0) {
-      sh.go[slot] = (uint32_t)got;
-      sh.task[slot] = task;
-      sh.phase[slot] = phase;
-      sh.tile[slot] = tile;
-    }
-    if (got == 1 && lane < (int)(sizeof(TaskBody) / 16)) {
-      const uint4 v = ld_cg_v4(reinterpret_cast<const uint4*>(&p.tasks[task].body) + lane);
-      reinterpret_cast<uint4*>(&sh.body[slot])[lane] = v;
-    }
-    __syncwarp();
-    if (lane == 0) sh.prof[kProfAcquire] += globaltimer() - t_acq;
-  };
-
-  if (warp == 0) claim(0, true);
-  __syncthreads();
+  // One claim, inlined once: with calls in this loop, or more copies of the
+  // claim, the product's inner loop spilled (1.7 to 2.0 ms instead of 1.5 for
+  // 16 x 16 products of 512^3).
+  bool have = false;  // slot cur holds a tile
   int cur = 0;
   while (true) {
-    if (sh.go[cur] != 1 || sh.abort) break;
     const int nxt = cur ^ 1;
-    const uint64_t t_tile = tid == 0 ? globaltimer() : 0;
     const TaskBody& b = sh.body[cur];
-    const uint32_t task = sh.task[cur], tile = sh.tile[cur];
-    int bucket = kProfVadd;
-    bool early = false;  // warp 0 claims the next tile while this one runs
-
-    if (b.type == kTaskVadd || b.type == kTaskVmul) {
-      const int64_t lo = (int64_t)tile * b.vadd_tile;
-      const int64_t hi = min(b.n, lo + b.vadd_tile);
-      if (warp == 0) {
-        claim(nxt, false);
-      } else if (b.type == kTaskVadd) {
-        vadd_range(reinterpret_cast<const float*>(b.a), reinterpret_cast<const float*>(b.b),
-                   reinterpret_cast<float*>(b.c), lo, hi, tid - 32, kThreads - 32);
-      } else {
-        vmul_range(reinterpret_cast<const float*>(b.a), reinterpret_cast<const float*>(b.b),
-                   reinterpret_cast<float*>(b.c), lo, hi, tid - 32, kThreads - 32, b.k);
-      }
-      early = true;
-    } else {
-      bucket = kProfGemm;
-      const int tm = (int)(tile / b.tiles_n), tn = (int)(tile % b.tiles_n);
+    const bool vec = have && (b.type == kTaskVadd || b.type == kTaskVmul);
+    if (tid == 0) sh.t_tile = globaltimer();
+    if (have && !vec) {
+      const uint32_t tile = sh.tile[cur];
       fma_tile(reinterpret_cast<const float*>(b.a), reinterpret_cast<const float*>(b.b),
-               reinterpret_cast<float*>(b.c), b.m, (int)b.n, b.k, tm, tn, reinterpret_cast<FmaSmem*>(dyn_smem));
+               reinterpret_cast<float*>(b.c), b.m, (int)b.n, b.k, (int)(tile / b.tiles_n), (int)(tile % b.tiles_n),
+               reinterpret_cast<FmaSmem*>(dyn_smem));
+      fma_finish(p, sh, cur, kProfGemm);  // before the claim, which may wait
     }
-    // need[cur]: the look-ahead claim found nothing, so warp 0 must claim
-    // (blocking) after this tile. Written before the barrier and not touched
-    // again until two tiles later, so every thread reads the same value (the
-    // blocking claim itself rewrites go[nxt] while others may still look).
-    if (warp == 0 && lane == 0) {
-      if (!early) sh.go[nxt] = 2;
-      sh.need[cur] = sh.go[nxt] == 2 ? 1u : 0u;
+    // Warp 0 claims the next tile: while the others run a vector tile (then
+    // without waiting), else waiting for one.
+    if (warp == 0) {
+      fma_claim(p, sh, nxt, !vec);
+    } else if (vec) {
+      const int64_t lo = (int64_t)sh.tile[cur] * b.vadd_tile;
+      const int64_t hi = min(b.n, lo + b.vadd_tile);
+      const float* x = reinterpret_cast<const float*>(b.a);
+      const float* y = reinterpret_cast<const float*>(b.b);
+      float* z = reinterpret_cast<float*>(b.c);
+      if (b.type == kTaskVadd) vadd_range<false, 8>(x, y, z, lo, hi, tid - 32, kFmaThreads - 32);
+      else vmul_range<false, 8>(x, y, z, lo, hi, tid - 32, kFmaThreads - 32, b.k);
     }
-    // Results written into host memory: visible to the host before the
-    // task's completion word.
-    if (b.flags & kFlagDirectOut)
-      __threadfence_system();
-    else
-      __threadfence();
-    __syncthreads();
-    if (sh.abort) {
-      if (tid == 0) report_error(p, kStatusTimeout, sh.fail_where, task);
-      break;
-    }
-    if (tid == 0) {
-      sh.prof[bucket] += globaltimer() - t_tile;
-      sh.prof[kProfTiles] += 1;
-      finish_tile(p, task, b.ntiles, b.tag, b.flags);
-    }
-    if (sh.need[cur]) {
-      // Nothing was claimable while the tile ran: wait for work now that its
-      // completion is published.
-      if (warp == 0) claim(nxt, true);
-      __syncthreads();
-    }
+    if (vec) fma_finish(p, sh, cur, kProfVadd);
+    else __syncthreads();
+    const uint32_t go = sh.go[nxt];  // not written again before the next barrier but one
+    if (go == 0) break;
+    have = go == 1;
     cur = nxt;
   }
   __syncthreads();
   if (tid == 0) sched_exit(p, sh.prof);
 }
 
-// ---------------------------------------------------------- split3 scheduler
+// ------------------------------------------------------------ pair scheduler
 //
-// Roles (see gvm_fused.cuh): warp kFzCtlWarp claims tiles and passes them to
-// the other warps through a ring of kFzItems items in shared memory; the MMA
-// warp and the converter warps each walk the ring in order. GEMM tiles run
-// through the fused split3 pipeline (the epilogue of a tile overlaps the
-// MMAs of the next); vector-add tiles run on the converter warps. No warp
-// waits for another warp's tile to finish except through the pipeline's own
-// barriers, so the next tile's claim, staging and MMAs overlap this one's.
+// The split3 scheduler on clusters of two CTAs (gvm_pair.cuh). The leader's
+// control warp claims tiles and posts each to the item rings of both CTAs;
+// every role of both walks the items in order. A GEMM tile is the pair's: the
+// CTAs stage their halves of the operands, the leader issues the MMAs, each
+// CTA's epilogue warps store its 128 rows. A vector tile is split in two
+// halves, each run by a CTA's converter and epilogue warps. Either way each
+// CTA counts its half, so a task is complete after 2 x ntiles counts. No warp
+// waits for another warp's tile except through the pipeline's barriers.
 
-constexpr int kFzItems = 4;
-constexpr uint32_t kItemExit = 0, kItemNop = 0xffu;  // besides the task types
-constexpr int kFinSlots = 16;  // per-item finish counters (items in flight < 16)
+constexpr int kItems = 4;                               // items in flight between the control warp and the others
+constexpr uint32_t kItemExit = 0, kItemNop = 0xffu;     // besides the task types
+constexpr int kFinSlots = 16;                           // per-item finish counters (items in flight < 16)
+constexpr int kPrVecThreads = (kPrEpiWarps + kPrConvWarps) * 32;
 
-// A staged GEMM tile whose accumulator is not drained yet.
-struct FzPend {
-  uint64_t c;
-  int64_t n;
-  int32_t m;
-  uint32_t tile, tiles_n, task, ntiles, tag, flags, seq;
-};
-
-struct FzItem {
-  uint32_t kind;  // kItemExit, kItemNop or a task type (kTaskVadd, kTaskSgemm, kTaskVmul)
+// An item: what to run, then the task's fields as they lie in the task table.
+struct alignas(16) PrItem {
+  uint32_t kind;  // kItemExit, kItemNop or a task type
   uint32_t task;
   uint32_t tile;
-  uint32_t tag;
-  uint32_t flags;
-  uint32_t ntiles;
-  uint32_t tiles_n;
+  uint32_t pad;
+  uint32_t type, flags, rank, slot;
+  uint32_t tag, ntiles, nsplit, tiles_m;
+  uint32_t tiles_n, kp;
   int32_t m;
   int32_t k;
-  uint32_t pad;
   int64_t n;
-  int64_t vadd_tile;
-  uint64_t a, b, c;
-  uint64_t tma;  // wide split3: device address of the task's A tensor map, or 0
+  int64_t span;  // vector tasks: elements per tile; SGEMM: columns per tile
+  uint64_t a, b, c, scratch;
 };
+constexpr int kItemFields = 6;  // 16-byte pieces of task fields
+static_assert(sizeof(PrItem) == 16 * (kItemFields + 1) && offsetof(TaskBody, c) - offsetof(TaskBody, type) ==
+                  offsetof(PrItem, c) - offsetof(PrItem, type), "item = header + task fields");
 
-// One thread: ask L2 for a GEMM item's task operands -- A's 128-row block
+// One thread: ask L2 for a GEMM item's task operands -- A's block of tile_m rows
 // of the tile's row (from the tile in column 0 of its row) and all of B
 // (from tile (0, 0)) -- so that each task's operands are requested once, in
 // pieces of at most 1 MiB, when they are 16-byte aligned, span a multiple
 // of 16 bytes and B holds at most 4 MiB. A hint only.
-__device__ __forceinline__ void prefetch_task_operands(const FzItem& it) {
+template <class Item>
+__device__ __forceinline__ void prefetch_task_operands(const Item& it, int64_t tile_m) {
   if (it.kind != kTaskSgemm || (it.k & 3) || ((it.a | it.b) & 15)) return;
   const uint32_t tm = it.tile / it.tiles_n, tn = it.tile % it.tiles_n;
   if (tn != 0) return;
@@ -696,43 +704,41 @@ __device__ __forceinline__ void prefetch_task_operands(const FzItem& it) {
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(addr + off), "r"((uint32_t)len) : "memory");
     }
   };
-  const int64_t rows = min((int64_t)kTcM, (int64_t)it.m - (int64_t)tm * kTcM);
-  if (rows > 0) pf(it.a + (uint64_t)tm * kTcM * (uint64_t)it.k * 4u, (uint64_t)rows * (uint64_t)it.k * 4u);
+  const int64_t rows = min(tile_m, (int64_t)it.m - (int64_t)tm * tile_m);
+  if (rows > 0) pf(it.a + (uint64_t)tm * (uint64_t)tile_m * (uint64_t)it.k * 4u, (uint64_t)rows * (uint64_t)it.k * 4u);
   const uint64_t b_bytes = (uint64_t)it.k * (uint64_t)it.n * 4u;
   if (tm == 0 && b_bytes <= (4u << 20) && (b_bytes & 15) == 0) pf(it.b, b_bytes);
 }
 
-// Shared state of a tensor-core scheduler CTA; Pipe is the tile form's
-// pipeline (FzShared: 128 x 256 tiles, WdShared: 256 x 256 tiles).
-template <class Pipe>
-struct alignas(128) TensorSchedShared {
-  Pipe fz;
-  uint64_t item_full[kFzItems];   // control -> consumers (1 arrival)
-  uint64_t item_empty[kFzItems];  // consumers -> control (converter warps + MMA warp)
-  FzItem items[kFzItems];
-  uint32_t fin[kFinSlots];        // converter warps done with item (seq % kFinSlots)
-  FzPend pend[kFzConvWarps][3];   // per converter warp: GEMM tiles by tile number % 3 (staged, not yet counted)
+struct PairSchedShared {
+  PrShared ps;
+  uint64_t item_full[kItems];   // each CTA: control -> its consumers
+  uint64_t item_empty[kItems];  // leader: consumers of both CTAs -> control
+  PrItem items[kItems];
+  uint32_t fin[kFinSlots];        // warps of this CTA done with item (seq % kFinSlots)
   uint32_t abort;
   uint32_t fail_where;
-  uint64_t prof[kProfSlots];  // kProf* counters; each slot written by one thread only
-  uint64_t claim[4];  // Claim state, owned by the control warp
+  uint64_t prof[kProfSlots];      // kProf* counters; each slot written by one thread only
+  uint64_t claim[4];              // Claim state, owned by the control warp
+  uint32_t list[2 * 32 * kMaxQuantum];  // ingest's scratch, control warp
+  uint64_t g_begin;               // %globaltimer and clock64 when the CTA began
+  long long c_begin;
 };
+constexpr uint32_t kPairSmemBytes = kPrRingBytes + sizeof(PairSchedShared);
+static_assert(kPairSmemBytes <= 227 * 1024, "pair form shared memory");
 
-// Records a failure seen by this CTA: the CTA flag stops its other warps'
-// waits, report_error stops the other CTAs and tells the host.
-template <class Sh>
-__device__ void cta_fail(const SchedParams& p, Sh& sh, uint32_t where, uint32_t info) {
-  sh.fail_where = where;
-  sh.abort = 1;
-  report_error(p, kStatusTimeout, where, info);
+__device__ __forceinline__ PrTile pair_tile(const PrItem& it) {
+  return pr_tile(reinterpret_cast<const float*>(it.a), reinterpret_cast<const float*>(it.b),
+                 reinterpret_cast<float*>(it.c), it.m, it.n, it.k, (int)(it.tile / it.tiles_n),
+                 (int)(it.tile % it.tiles_n), (int)it.span, (it.flags / kFlagTmA) & 15u);
 }
+static_assert(kFlagTmB == 2 * kFlagTmA && kFlagPackA == 4 * kFlagTmA && kFlagPackB == 8 * kFlagTmA,
+              "map flags are PrTile::land bits");
 
-// A converter warp has written its share of item `seq` (a vector-add range or
-// a drained accumulator). The last of the kFzConvWarps warps completes the
-// tile. Lanes fence their own stores before lane 0 counts the warp.
-template <class Sh>
-__device__ void conv_item_done(const SchedParams& p, Sh& sh, uint32_t seq, uint32_t task, uint32_t ntiles,
-                               uint32_t tag, uint32_t flags) {
+// One warp has written its share of an item (`warps` share it in this CTA):
+// the last one counts this CTA's half of the tile.
+__device__ __forceinline__ void pair_item_done(const SchedParams& p, PairSchedShared& sh, uint32_t seq, uint32_t warps,
+                                               uint32_t task, uint32_t ntiles, uint32_t tag, uint32_t flags) {
   // Results written into host memory must be visible to the host before the
   // task's completion word is.
   if (flags & kFlagDirectOut)
@@ -742,387 +748,357 @@ __device__ void conv_item_done(const SchedParams& p, Sh& sh, uint32_t seq, uint3
   __syncwarp();
   if ((threadIdx.x & 31) == 0) {
     uint32_t* f = &sh.fin[seq % kFinSlots];
-    if (atomicAdd(f, 1u) == kFzConvWarps - 1) {
+    if (atomicAdd(f, 1u) == warps - 1) {
       *f = 0;
       __threadfence();
-      finish_tile(p, task, ntiles, tag, flags);
+      finish_tile(p, task, 2 * ntiles, tag, flags);
     }
   }
   __syncwarp();
 }
 
-// The split3 scheduler CTA for either tile form (kWide: 256 x 256 tiles).
-enum : int { kFormFused = 0, kFormWide = 1, kFormTma = 2 };
+// A consumer's next item, for one thread or (kWarp) a whole warp; false when
+// the wait ran out or the CTA stopped.
+template <bool kWarp>
+__device__ __forceinline__ bool pair_item_wait(const SchedParams& p, PairSchedShared& sh, uint32_t seq) {
+  uint64_t* bar = &sh.item_full[seq % kItems];
+  const uint32_t ph = (seq / kItems) & 1u;
+  if (kWarp ? mbar_wait_warp<true>(bar, ph, p.wait_timeout_ns, &sh.abort)
+            : mbar_wait_cluster(bar, ph, p.wait_timeout_ns, &sh.abort))
+    return true;
+  if (!sh.abort) {
+    pr_fail(&sh.ps, &sh.abort, &sh.fail_where, kWhereItemWait);
+    report_error(p, kStatusTimeout, kWhereItemWait, seq);
+  }
+  return false;
+}
+__device__ __forceinline__ void pair_item_release(PairSchedShared& sh, uint32_t seq) {
+  mbar_arrive_cta(&sh.item_empty[seq % kItems], 0);
+}
 
-template <int kForm>
-__device__ __forceinline__ void sched_tc_body(const SchedParams& p) {
-  constexpr bool kWide = kForm == kFormWide;
-  constexpr bool kTma = kForm == kFormTma;
-  using Pipe = typename std::conditional<kWide, WdShared,
-                                         typename std::conditional<kTma, TmShared, FzShared>::type>::type;
-  __shared__ TensorSchedShared<Pipe> sh;
-  extern __shared__ uint8_t dyn_smem[];
-  uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dyn_smem) + 1023) & ~uintptr_t(1023));
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+// The roles, each a function of its own: ptxas gives a function the registers
+// that its callers do not hold, and what spills is read back from L2 (the
+// control warp's acquires keep invalidating L1). With the roles inlined into
+// the kernel the converters' loop spilled and a 512^3 launch took 1.6 ms.
+#define PAIR_ROLE static __device__ __noinline__ void
+
+// Control (leader): claims tiles into both item rings.
+PAIR_ROLE pair_control(const SchedParams& p, PairSchedShared& sh) {
+  const int lane = threadIdx.x & 31;
   Claim* cl = reinterpret_cast<Claim*>(sh.claim);
+  const uint64_t to = p.wait_timeout_ns;
+  for (uint32_t seq = 0;; ++seq) {
+    const uint32_t slot = seq % kItems, ph = (seq / kItems) & 1u;
+    uint32_t ok = 1;
+    if (lane == 0) ok = mbar_wait_cluster(&sh.item_empty[slot], ph ^ 1u, to, &sh.abort) ? 1u : 0u;
+    if (!__shfl_sync(0xffffffffu, ok, 0)) {
+      if (lane == 0 && !sh.abort) {
+        pr_fail(&sh.ps, &sh.abort, &sh.fail_where, kWhereItemRing);
+        report_error(p, kStatusTimeout, kWhereItemRing, seq);
+      }
+      break;
+    }
+    const uint64_t t0 = globaltimer();
+    uint32_t task = 0, tile = 0;
+    // An idle control warp posts a no-op item now and then, so that the
+    // other warps' waits for items stay bounded.
+    const int got = sh.abort ? 0 : acquire<true>(p, cl, sh.list, task, tile, sh.prof, true, to / 4);
+    // Lanes 0..5 carry the task's fields, lane 6 the header (it reads the piece
+    // that begins with the type), to both CTAs.
+    if (lane <= kItemFields) {
+      uint4 v = make_uint4(got == 2 ? kItemNop : kItemExit, 0, 0, 0);
+      if (got == 1)
+        v = ld_cg_v4(reinterpret_cast<const uint8_t*>(&p.tasks[task].body) + kFieldsAt + 16 * (lane % kItemFields));
+      if (lane == kItemFields && got == 1) v = make_uint4(v.x, task, tile, 0);
+      uint4* dst = reinterpret_cast<uint4*>(&sh.items[slot]) + (lane == kItemFields ? 0 : lane + 1);
+      *dst = v;
+      st_cluster_v4(mapa_shared(smem_u32(dst), 1), v);
+      mbar_arrive_release_cta(&sh.item_full[slot], 1);
+      mbar_arrive(&sh.item_full[slot]);
+    }
+    __syncwarp();
+    if (lane == 0) {
+      sh.prof[kProfAcquire] += globaltimer() - t0;
+      // L2 prefetch, a few tiles ahead of the producers: the item two claims
+      // back (its slot is rewritten only two claims from now).
+      if (p.prefetch && seq >= 2) prefetch_task_operands(sh.items[(seq + 2) % kItems], kPrM);
+    }
+    __syncwarp();
+    if (got == 0) break;
+  }
+}
+
+// This CTA's half of a vector item.
+struct PairVec {
+  const float* a;
+  const float* b;
+  float* c;
+  int64_t len;
+};
+__device__ __forceinline__ PairVec pair_vec(const PrItem& it, uint32_t cta) {
+  const int64_t half = it.span / 2, lo = (int64_t)it.tile * it.span + (int64_t)cta * half;
+  const int64_t len = min(it.n - lo, half);
+  return PairVec{reinterpret_cast<const float*>(it.a) + lo, reinterpret_cast<const float*>(it.b) + lo,
+                 reinterpret_cast<float*>(it.c) + lo, len > 0 ? len : 0};
+}
+// Vector items whose operands bulk copies can address run through the landing
+// ring (the halves of a tile begin at multiples of 512 elements).
+__device__ __forceinline__ bool pair_vec_lands(const PrItem& it) { return ((it.a | it.b) & 15) == 0; }
+
+// MMA issue (leader, one thread): GEMM items only; every item is read and released.
+PAIR_ROLE pair_mma(const SchedParams& p, PairSchedShared& sh, uint8_t* stages) {
+  uint32_t it_k = 0, tile_no = 0;
+  for (uint32_t seq = 0; pair_item_wait<false>(p, sh, seq); ++seq) {
+    const PrItem& item = sh.items[seq % kItems];
+    const uint32_t kind = item.kind;
+    const PrTile t = kind == kTaskSgemm ? pair_tile(item) : PrTile{};
+    pair_item_release(sh, seq);
+    if (kind == kItemExit) break;
+    if (kind != kTaskSgemm) continue;
+    if (!pr_mma(t, stages, &sh.ps, it_k, tile_no, p.wait_timeout_ns, &sh.abort, &sh.fail_where,
+                &sh.prof[kProfMmaWait])) {
+      report_error(p, kStatusTimeout, sh.fail_where, seq);
+      break;
+    }
+    it_k += (uint32_t)((t.k + kTcBK - 1) / kTcBK);
+    ++tile_no;
+  }
+}
+
+// Producer (one thread): the tensor copies of every GEMM item's k-steps, the
+// bulk copies of vector items.
+PAIR_ROLE pair_produce(const SchedParams& p, PairSchedShared& sh, uint8_t* land) {
+  uint32_t it_l = 0, pend = 0;
+  for (uint32_t seq = 0; pair_item_wait<false>(p, sh, seq); ++seq) {
+    const PrItem& item = sh.items[seq % kItems];
+    const uint32_t kind = item.kind;
+    const CUtensorMap* tm = &p.tasks[item.task].body.tmA;
+    const PrTile t = kind == kTaskSgemm ? pair_tile(item) : PrTile{};
+    const bool vec = (kind == kTaskVadd || kind == kTaskVmul) && pair_vec_lands(item);
+    const PairVec v = vec ? pair_vec(item, sh.ps.cta) : PairVec{};
+    pair_item_release(sh, seq);
+    if (kind == kItemExit) break;
+    if (kind != kTaskSgemm && !vec) continue;
+    // The operands may have been written by this kernel's own stores, and
+    // the maps were written by the ingest's.
+    fence_proxy_async_global();
+    bool ok;
+    if (vec) {
+      ok = pr_vec_produce(v.a, v.b, v.len, land, &sh.ps, it_l, p.wait_timeout_ns, &sh.abort, &sh.fail_where, pend);
+      it_l += pr_vec_chunks(v.len);
+    } else {
+      if (t.land & kPrMapA) fence_tensormap_acquire(tm);
+      if (t.land & kPrMapB) fence_tensormap_acquire(tm + 1);
+      ok = pr_produce(t, land, &sh.ps, it_l, tm, tm + 1, p.wait_timeout_ns, &sh.abort, &sh.fail_where, pend);
+      it_l += (uint32_t)((t.k + kTcBK - 1) / kTcBK);
+    }
+    if (!ok) {
+      report_error(p, kStatusTimeout, sh.fail_where, seq);
+      break;
+    }
+  }
+  pr_produce_quiesce(&sh.ps, pend, p.wait_timeout_ns);
+}
+
+// Vector item without 16-byte aligned operands, converter and epilogue warps
+// together, by direct loads.
+__device__ __forceinline__ void pair_vector(const SchedParams& p, PairSchedShared& sh, uint32_t seq) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const PrItem& item = sh.items[seq % kItems];
+  const uint32_t kind = item.kind, task = item.task, ntiles = item.ntiles, tag = item.tag, flags = item.flags;
+  const int iters = item.k;
+  const PairVec v = pair_vec(item, sh.ps.cta);
+  __syncwarp();
+  if (lane == 0) pair_item_release(sh, seq);
+  if (kind == kTaskVmul) vmul_range<true>(v.a, v.b, v.c, 0, v.len, tid, kPrVecThreads, iters);
+  else vadd_range<true>(v.a, v.b, v.c, 0, v.len, tid, kPrVecThreads);
+  pair_item_done(p, sh, seq, kPrEpiWarps + kPrConvWarps, task, ntiles, tag, flags);
+}
+
+// Converter warps: stage GEMM tiles, run vector tiles.
+PAIR_ROLE pair_convert(const SchedParams& p, PairSchedShared& sh, uint8_t* land, uint8_t* stages) {
+  const int lane = threadIdx.x & 31;
+  const bool prof = threadIdx.x == kPrConvWarp0 * 32;
+  uint32_t it_k = 0, it_l = 0;
+  for (uint32_t seq = 0; pair_item_wait<true>(p, sh, seq); ++seq) {
+    const PrItem& item = sh.items[seq % kItems];
+    const uint32_t kind = item.kind;
+    const uint64_t t0 = prof ? globaltimer() : 0;
+    bool ok = true;
+    if (kind == kTaskSgemm) {
+      const PrTile t = pair_tile(item);
+      __syncwarp();
+      if (lane == 0) pair_item_release(sh, seq);
+      ok = pr_convert(t, land, stages, &sh.ps, it_k, it_l, p.wait_timeout_ns, &sh.abort, &sh.fail_where);
+      const uint32_t nkb = (uint32_t)((t.k + kTcBK - 1) / kTcBK);
+      it_k += nkb;
+      it_l += nkb;
+      if (prof) sh.prof[kProfGemm] += globaltimer() - t0;
+    } else if (kind == kTaskVadd || kind == kTaskVmul) {
+      if (pair_vec_lands(item)) {
+        const uint32_t task = item.task, ntiles = item.ntiles, tag = item.tag, flags = item.flags;
+        const int iters = item.k;
+        const PairVec v = pair_vec(item, sh.ps.cta);
+        __syncwarp();
+        if (lane == 0) pair_item_release(sh, seq);
+        ok = kind == kTaskVmul ? pr_vec_convert<kElemMul>(v.a, v.b, v.c, v.len, iters, land, &sh.ps, it_l,
+                                                          p.wait_timeout_ns, &sh.abort, &sh.fail_where)
+                               : pr_vec_convert<kElemAdd>(v.a, v.b, v.c, v.len, 0, land, &sh.ps, it_l,
+                                                          p.wait_timeout_ns, &sh.abort, &sh.fail_where);
+        it_l += pr_vec_chunks(v.len);
+        if (ok) pair_item_done(p, sh, seq, kPrConvWarps, task, ntiles, tag, flags);
+      } else {
+        pair_vector(p, sh, seq);
+      }
+      if (prof) {
+        sh.prof[kProfVadd] += globaltimer() - t0;
+        if (sh.ps.cta == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&sh.prof[kProfTiles]), 1ull);
+      }
+    } else {
+      __syncwarp();
+      if (lane == 0) pair_item_release(sh, seq);
+      if (kind == kItemExit) break;
+    }
+    if (!ok) {
+      if (lane == 0) report_error(p, kStatusTimeout, sh.fail_where, 0);
+      break;
+    }
+  }
+}
+
+// Epilogue warps: store GEMM tiles and count them.
+PAIR_ROLE pair_epilogue(const SchedParams& p, PairSchedShared& sh) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  uint32_t tile_no = 0;
+  for (uint32_t seq = 0; pair_item_wait<true>(p, sh, seq); ++seq) {
+    const PrItem& item = sh.items[seq % kItems];
+    const uint32_t kind = item.kind;
+    if ((kind == kTaskVadd || kind == kTaskVmul) && !pair_vec_lands(item)) {
+      pair_vector(p, sh, seq);
+      continue;
+    }
+    const uint32_t task = item.task, ntiles = item.ntiles, tag = item.tag, flags = item.flags;
+    const PrTile t = kind == kTaskSgemm ? pair_tile(item) : PrTile{};
+    __syncwarp();
+    if (lane == 0) pair_item_release(sh, seq);
+    if (kind == kItemExit) break;
+    if (kind != kTaskSgemm) continue;
+    const uint64_t t0 = pr_epilogue(t, &sh.ps, tile_no, p.wait_timeout_ns, &sh.abort, &sh.fail_where);
+    if (t0 == 0) {
+      if (lane == 0) report_error(p, kStatusTimeout, sh.fail_where, 0);
+      break;
+    }
+    pair_item_done(p, sh, seq, kPrEpiWarps, task, ntiles, tag, flags);
+    if (tid == 0) {
+      sh.prof[kProfEpilogue] += globaltimer() - t0;
+      if (sh.ps.cta == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&sh.prof[kProfTiles]), 1ull);
+    }
+    ++tile_no;
+  }
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPrThreads, 1)
+    sched_pair_kernel(const __grid_constant__ SchedParams p) {
+  extern __shared__ __align__(1024) uint8_t dyn_smem[];
+  uint8_t* land = dyn_smem;
+  uint8_t* stages = dyn_smem + kPrLand * kPrLandBytes;
+  PairSchedShared& sh = *reinterpret_cast<PairSchedShared*>(dyn_smem + kPrRingBytes);
+  const int tid = threadIdx.x, warp = tid >> 5;
   if (tid == 0) {
     sh.abort = 0;
     sh.fail_where = 0;
+    sh.g_begin = globaltimer();
+    sh.c_begin = clock64();
     for (int i = 0; i < kProfSlots; ++i) sh.prof[i] = 0;
     for (int i = 0; i < kFinSlots; ++i) sh.fin[i] = 0;
-    for (int i = 0; i < kFzItems; ++i) {
-      mbar_init(&sh.item_full[i], 1);
-      mbar_init(&sh.item_empty[i], kFzConvWarps + (kTma ? 2 : 1));  // converters, MMA (and producer)
+    for (int i = 0; i < kItems; ++i) {
+      mbar_init(&sh.item_full[i], kItemFields + 1);  // a lane per 16-byte piece
+      // Each CTA's epilogue and converter warps and producer; the leader's MMA thread.
+      mbar_init(&sh.item_empty[i], 2 * (kPrEpiWarps + kPrConvWarps + 1) + 1);
     }
+    Claim* cl = reinterpret_cast<Claim*>(sh.claim);
     cl->has_resv = 0;
     cl->stall_since = 0;
     cl->hint = ld_relaxed_gpu64(&p.ctrl->first_entry);
     sched_enter(p);
   }
-  // initialises the pipeline barriers, fences all inits, allocates TMEM
-  if constexpr (kWide)
-    wd_init(&sh.fz);
-  else if constexpr (kTma)
-    tm_init(&sh.fz);
-  else
-    fz_init(&sh.fz);
-
-  if (warp == kFzCtlWarp) {
-    // ---- control: claim tiles into the item ring.
-    for (uint32_t seq = 0;; ++seq) {
-      const uint32_t slot = seq % kFzItems, ph = (seq / kFzItems) & 1u;
-      uint32_t ok = 1;
-      if (lane == 0) ok = mbar_wait(&sh.item_empty[slot], ph ^ 1u, p.wait_timeout_ns, &sh.abort) ? 1u : 0u;
-      if (!__shfl_sync(0xffffffffu, ok, 0)) {
-        if (lane == 0 && !sh.abort) cta_fail(p, sh, kWhereItemRing, seq);
-        break;
-      }
-      const uint64_t t0 = globaltimer();
-      uint32_t task = 0, phase = 0, tile = 0;
-      // An idle control warp posts a no-op item now and then, so that the
-      // other warps' waits for items stay bounded.
-      const int got = sh.abort ? 0 : acquire<true>(p, cl, task, phase, tile, sh.prof, true, p.wait_timeout_ns / 4);
-      if (lane == 0) {
-        FzItem& it = sh.items[slot];
-        it.kind = got == 1 ? 0u : (got == 2 ? kItemNop : kItemExit);
-        if (got == 1) {
-          const TaskBody* b = &p.tasks[task].body;
-          it.kind = __ldcg(&b->type);
-          it.task = task;
-          it.tile = tile;
-          it.tag = __ldcg(&b->tag);
-          it.flags = __ldcg(&b->flags);
-          it.ntiles = __ldcg(&b->ntiles);
-          it.tiles_n = __ldcg(&b->tiles_n);
-          it.m = __ldcg(&b->m);
-          it.k = __ldcg(&b->k);
-          it.n = __ldcg(&b->n);
-          it.vadd_tile = __ldcg(&b->vadd_tile);
-          it.tma = (it.flags & kFlagTmA) ? reinterpret_cast<uint64_t>(&b->tmA) : 0ull;
-          it.a = __ldcg(&b->a);
-          it.b = __ldcg(&b->b);
-          it.c = __ldcg(&b->c);
-        }
-        sh.prof[kProfAcquire] += globaltimer() - t0;
-        mbar_arrive(&sh.item_full[slot]);
-        // L2 prefetch, a few tiles ahead of the staging warps: the item two
-        // claims back (its slot is rewritten only two claims from now).
-        if (p.prefetch && seq >= 2) prefetch_task_operands(sh.items[(seq + 2) % kFzItems]);
-      }
-      __syncwarp();
-      if (got == 0) break;
+  pr_init(&sh.ps);  // the pipeline's barriers, fences all inits, TMEM
+  const bool leader = sh.ps.cta == 0;
+  if (warp < kPrEpiWarps) {
+    pair_epilogue(p, sh);
+  } else if (warp < kPrMmaWarp) {
+    pair_convert(p, sh, land, stages);
+  } else if (warp == kPrMmaWarp) {
+    if (leader && elect_one()) {
+      pair_mma(p, sh, stages);
+      umma_commit_pair(&sh.ps.mma_done);
     }
-  } else if (warp == kFzMmaWarp) {
-    // ---- MMA issue: GEMM items only; every item is read and released.
-    uint32_t it_k = 0, tile_no = 0;
-    for (uint32_t seq = 0;; ++seq) {
-      const uint32_t slot = seq % kFzItems, ph = (seq / kFzItems) & 1u;
-      if (!mbar_wait(&sh.item_full[slot], ph, p.wait_timeout_ns, &sh.abort)) {
-        if (lane == 0 && !sh.abort) cta_fail(p, sh, kWhereItemWait, seq);
-        break;
-      }
-      const FzItem& item = sh.items[slot];
-      const uint32_t kind = item.kind;
-      FzTile t{reinterpret_cast<const float*>(item.a), reinterpret_cast<const float*>(item.b),
-               reinterpret_cast<float*>(item.c), item.n, item.m, item.k, 0, 0};
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sh.item_empty[slot]);
-      if (kind == kItemExit) break;
-      if (kind != kTaskSgemm) continue;
-      uint32_t ok = 1;
-      if (lane == 0) {
-        if constexpr (kWide)
-          ok = wd_mma(t, stages, &sh.fz, it_k, tile_no, p.wait_timeout_ns, &sh.abort, &sh.fail_where,
-                      &sh.prof[kProfMmaWait])
-                   ? 1u
-                   : 0u;
-        else if constexpr (kTma)
-          ok = tm_mma(t, stages, &sh.fz, it_k, tile_no, p.wait_timeout_ns, &sh.abort, &sh.fail_where,
-                      &sh.prof[kProfMmaWait])
-                   ? 1u
-                   : 0u;
-        else
-          ok = fz_mma(t, stages, &sh.fz, it_k, tile_no, p.wait_timeout_ns, &sh.abort, &sh.fail_where,
-                      &sh.prof[kProfMmaWait])
-                   ? 1u
-                   : 0u;
-      }
-      if (!__shfl_sync(0xffffffffu, ok, 0)) {
-        if (lane == 0) report_error(p, kStatusTimeout, sh.fail_where, seq);
-        break;
-      }
-      it_k += (uint32_t)((t.k + kTcBK - 1) / kTcBK);
-      ++tile_no;
-    }
-  } else if (kTma && warp == kTmProducerWarp) {
-    // ---- producer (TMA form): every GEMM item's k-steps, in order, get
-    // their stage once the MMAs release it, with the tensor copies of A and
-    // B when the task has maps.
-    if constexpr (kTma) {
-      uint32_t it_k = 0, pend[kTcStages] = {0, 0, 0, 0};
-      for (uint32_t seq = 0;; ++seq) {
-        const uint32_t slot = seq % kFzItems, ph = (seq / kFzItems) & 1u;
-        if (!mbar_wait(&sh.item_full[slot], ph, p.wait_timeout_ns, &sh.abort)) {
-          if (lane == 0 && !sh.abort) cta_fail(p, sh, kWhereItemWait, seq);
-          break;
-        }
-        const FzItem& item = sh.items[slot];
-        const uint32_t kind = item.kind;
-        const FzTile t{reinterpret_cast<const float*>(item.a), reinterpret_cast<const float*>(item.b),
-                       reinterpret_cast<float*>(item.c), item.n, item.m, item.k,
-                       (int)(kind == kTaskSgemm ? item.tile / item.tiles_n : 0),
-                       (int)(kind == kTaskSgemm ? item.tile % item.tiles_n : 0)};
-        const bool maps = (item.flags & (kFlagTmA | kFlagTmB)) == (kFlagTmA | kFlagTmB);
-        const CUtensorMap* tmA = maps ? reinterpret_cast<const CUtensorMap*>(item.tma) : nullptr;
-        const CUtensorMap* tmB = maps ? reinterpret_cast<const CUtensorMap*>(item.tma + sizeof(CUtensorMap)) : nullptr;
-        const bool b3 = (item.flags & kFlagTmB3) != 0;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.item_empty[slot]);
-        if (kind == kItemExit) break;
-        if (kind != kTaskSgemm) continue;
-        uint32_t ok = 1;
-        if (lane == 0) {
-          if (tmA != nullptr) {
-            // The maps were written by the ingest's generic stores.
-            fence_tensormap_acquire(tmA);
-            fence_tensormap_acquire(tmB);
-          }
-          ok = tm_produce(t, stages, &sh.fz, it_k, tmA, tmB, b3, p.wait_timeout_ns,
-                          &sh.abort, &sh.fail_where, pend)
-                   ? 1u
-                   : 0u;
-        }
-        if (!__shfl_sync(0xffffffffu, ok, 0)) {
-          if (lane == 0) report_error(p, kStatusTimeout, sh.fail_where, seq);
-          break;
-        }
-        it_k += (uint32_t)((t.k + kTcBK - 1) / kTcBK);
-      }
-      if (lane == 0) tm_quiesce(&sh.fz, pend, p.wait_timeout_ns);
-      __syncwarp();
-    }
-  } else if (warp < kFzConvWarps) {
-    // ---- converters: stage GEMM tiles; after staging tile T, count tile
-    // T-2 as finished (its stores were issued a tile ago, so the fence that
-    // orders them before the count hardly waits) and drain tile T-1's
-    // accumulator into C. Vector-add tiles, no-op items, the exit and an
-    // empty item ring flush both steps first, so that no completion waits
-    // for later work.
-    uint32_t it_k = 0, tile_no = 0;
-    bool has_drain = false, has_done = false;  // tile tile_no-1 to drain; tile done_no to count
-    uint32_t done_no = 0;
-    uint32_t land_n = 0, land_iss = 0;  // wide form: A landings this warp's group consumed, issued
-    // GEMM tile number i of this CTA is kept (by lane 0) in pend[warp][i % 3]
-    // until it is counted, out of the registers the staging loop needs.
-    auto tile_of = [](const FzItem& item) {
-      return FzTile{reinterpret_cast<const float*>(item.a), reinterpret_cast<const float*>(item.b),
-                    reinterpret_cast<float*>(item.c), item.n, item.m, item.k,
-                    (int)(item.tile / item.tiles_n), (int)(item.tile % item.tiles_n)};
-    };
-    auto count_done = [&]() {
-      if (!has_done) return;
-      const FzPend& d = sh.pend[warp][done_no % 3u];
-      conv_item_done(p, sh, d.seq, d.task, d.ntiles, d.tag, d.flags);
-      has_done = false;
-    };
-    auto drain = [&]() -> bool {
-      if (!has_drain) return true;
-      const uint64_t t0 = tid == 0 ? globaltimer() : 0;
-      const uint32_t no = tile_no - 1;
-      const FzPend& d = sh.pend[warp][no % 3u];
-      const FzTile pt{nullptr, nullptr, reinterpret_cast<float*>(d.c), d.n, d.m, 0, (int)(d.tile / d.tiles_n),
-                      (int)(d.tile % d.tiles_n)};
-      bool drained;
-      if constexpr (kWide)
-        drained = wd_epilogue(pt, &sh.fz, no, p.wait_timeout_ns, &sh.abort, &sh.fail_where);
-      else if constexpr (kTma)
-        drained = fz_epilogue(pt, &sh.fz.fz, no, p.wait_timeout_ns, &sh.abort, &sh.fail_where);
-      else
-        drained = fz_epilogue(pt, &sh.fz, no, p.wait_timeout_ns, &sh.abort, &sh.fail_where);
-      if (!drained) return false;
-      has_drain = false;
-      has_done = true;
-      done_no = no;
-      if (tid == 0) sh.prof[kProfEpilogue] += globaltimer() - t0;
-      return true;
-    };
-    auto flush = [&]() -> bool {
-      count_done();
-      if (!drain()) return false;
-      count_done();
-      return true;
-    };
-    bool ok = true;
-    for (uint32_t seq = 0;; ++seq) {
-      const uint32_t slot = seq % kFzItems, ph = (seq / kFzItems) & 1u;
-      if ((has_drain || has_done) && !mbar_try_wait(&sh.item_full[slot], ph)) {
-        ok = flush();  // nothing queued: finish what is pending before waiting
-        if (!ok) break;
-      }
-      if (!mbar_wait(&sh.item_full[slot], ph, p.wait_timeout_ns, &sh.abort)) {
-        if (lane == 0 && !sh.abort) cta_fail(p, sh, kWhereItemWait, seq);
-        ok = false;
-        break;
-      }
-      const FzItem& item = sh.items[slot];
-      const uint32_t kind = item.kind;
-      if (kind == kItemExit || kind == kItemNop) {
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.item_empty[slot]);
-        if (kind == kItemExit) break;
-        ok = flush();
-        if (!ok) break;
-        continue;
-      }
-      const uint64_t t0 = tid == 0 ? globaltimer() : 0;
-      if (kind == kTaskSgemm) {
-        const FzTile t = tile_of(item);
-        const CUtensorMap* tma = kWide ? reinterpret_cast<const CUtensorMap*>(item.tma) : nullptr;
-        const uint32_t item_flags = item.flags;
-        __syncwarp();
-        if (lane == 0) {
-          // The item's sequence number names its finish counter.
-          sh.pend[warp][tile_no % 3u] = FzPend{item.c, item.n, item.m, item.tile, item.tiles_n,
-                                               item.task, item.ntiles, item.tag, item.flags, seq};
-          mbar_arrive(&sh.item_empty[slot]);
-        }
-        __syncwarp();
-        if constexpr (kWide) {
-          // One accumulator: drain tile T-1 right after this group's first
-          // k-step of T (T's MMAs wait for it), then count T-1.
-          // The map was written by the ingest's generic stores: order them
-          // before the tensor copies that read it.
-          if (tma != nullptr && (warp % kFzGroupWarps) == 0) fence_tensormap_acquire(tma);
-          ok = wd_convert(t, stages, &sh.fz, it_k, p.wait_timeout_ns, &sh.abort, &sh.fail_where,
-                          tid == 0 ? &sh.prof[kProfStageWait] : nullptr, [&]() -> bool { return drain(); },
-                          land_n, land_iss, tma);
-          if (ok) ok = drain();  // the group had no k-step of T
-          if (ok) count_done();
-        } else if constexpr (kTma) {
-          const bool landed = (item_flags & (kFlagTmA | kFlagTmB)) == (kFlagTmA | kFlagTmB);
-          ok = tm_convert(t, stages, &sh.fz, it_k, landed, p.wait_timeout_ns, &sh.abort, &sh.fail_where,
-                          tid == 0 ? &sh.prof[kProfStageWait] : nullptr);
-          if (ok) {
-            count_done();
-            ok = drain();
-          }
-        } else {
-          ok = fz_convert<true>(t, stages, &sh.fz, it_k, p.wait_timeout_ns, &sh.abort, &sh.fail_where,
-                                tid == 0 ? &sh.prof[kProfStageWait] : nullptr);
-          if (ok) {
-            count_done();
-            ok = drain();
-          }
-        }
-        it_k += (uint32_t)((t.k + kTcBK - 1) / kTcBK);
-        has_drain = true;
-        ++tile_no;
-        if (tid == 0) sh.prof[kProfGemm] += globaltimer() - t0;
-      } else {  // vector add or vector multiply
-        const uint32_t task = item.task, ntiles = item.ntiles, tag = item.tag, flags = item.flags;
-        const int iters = item.k;
-        const int64_t lo = (int64_t)item.tile * item.vadd_tile;
-        const int64_t hi = min(item.n, lo + item.vadd_tile);
-        const float* a = reinterpret_cast<const float*>(item.a);
-        const float* b = reinterpret_cast<const float*>(item.b);
-        float* c = reinterpret_cast<float*>(item.c);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.item_empty[slot]);
-        ok = flush();
-        if (ok) {
-          if (kind == kTaskVmul) vmul_range(a, b, c, lo, hi, tid, kFzConvThreads, iters);
-          else vadd_range(a, b, c, lo, hi, tid, kFzConvThreads);
-          conv_item_done(p, sh, seq, task, ntiles, tag, flags);
-        }
-        if (tid == 0) sh.prof[kProfVadd] += globaltimer() - t0;
-      }
-      if (tid == 0) sh.prof[kProfTiles] += 1;
-      if (!ok) break;
-    }
-    if (ok && !sh.abort) ok = flush();
-    if (!ok && lane == 0) report_error(p, kStatusTimeout, sh.fail_where, 0);
-    if constexpr (kWide) wd_land_quiesce(&sh.fz, land_n, land_iss, p.wait_timeout_ns);
+  } else if (warp == kPrProdWarp) {
+    if (elect_one()) pair_produce(p, sh, land);
+  } else if (leader) {
+    pair_control(p, sh);
   }
-  if constexpr (kWide)
-    wd_teardown(&sh.fz);
-  else if constexpr (kTma)
-    fz_teardown(&sh.fz.fz);
-  else
-    fz_teardown(&sh.fz);
-  if (tid == 0) sched_exit(p, sh.prof);
-}
-
-__global__ void __launch_bounds__(kFzThreads, 1) sched_fused_kernel(const SchedParams p) {
-  sched_tc_body<kFormFused>(p);
-}
-
-__global__ void __launch_bounds__(kFzThreads, 1) sched_wide_kernel(const SchedParams p) {
-  sched_tc_body<kFormWide>(p);
-}
-
-__global__ void __launch_bounds__(kTmThreads, 1) sched_tma_kernel(const SchedParams p) {
-  sched_tc_body<kFormTma>(p);
+  __syncwarp();
+  pr_teardown(&sh.ps, 2 * p.wait_timeout_ns);
+  if (tid == 0) {
+    // The waits for k-steps were summed in SM clocks: to nanoseconds.
+    const double ns = (double)(globaltimer() - sh.g_begin) / (double)max(1ll, clock64() - sh.c_begin);
+    sh.prof[kProfMmaWait] = (uint64_t)(ns * (double)sh.prof[kProfMmaWait]);
+    sched_exit(p, sh.prof);
+  }
 }
 
 static size_t dyn_smem_bytes(int path) {
-  if (path == kPathSplit3 || path == kPathSplit3Tma) return (size_t)kTcStages * kTcStageBytes + 1024;
-  if (path == kPathSplit3Wide) return (size_t)kWdSmemBytes + 1024;
+  if (path == kPathSplit3) return kPairSmemBytes;
   return sizeof(FmaSmem) + 1024;
 }
 
 static const void* sched_fn(int path) {
-  if (path == kPathSplit3) return (const void*)sched_fused_kernel;
-  if (path == kPathSplit3Wide) return (const void*)sched_wide_kernel;
-  if (path == kPathSplit3Tma) return (const void*)sched_tma_kernel;
+  if (path == kPathSplit3) return (const void*)sched_pair_kernel;
   return (const void*)sched_fma_kernel;
 }
 
 static int sched_threads(int path) {
-  return path == kPathFma ? kThreads : path == kPathSplit3Tma ? kTmThreads : kFzThreads;
+  return path == kPathFma ? kFmaThreads : kPrThreads;
 }
 
-cudaError_t scheduler_setup(int path, int* blocks_per_sm, size_t* smem_bytes) {
+cudaError_t scheduler_setup(int path, int sms, int* max_ctas, size_t* smem_bytes) {
   const size_t smem = dyn_smem_bytes(path);
   const void* fn = sched_fn(path);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
+  if (path == kPathSplit3) {
+    // As many clusters of two CTAs as the device holds at once.
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(2);
+    c.blockDim = dim3(kPrThreads);
+    c.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 2;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    c.attrs = &attr;
+    c.numAttrs = 1;
+    int clusters = 0;
+    e = cudaOccupancyMaxActiveClusters(&clusters, fn, &c);
+    if (e != cudaSuccess) return e;
+    *max_ctas = 2 * clusters;
+    *smem_bytes = smem;
+    return cudaSuccess;
+  }
   int nb = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, sched_threads(path), smem);
   if (e != cudaSuccess) return e;
-  *blocks_per_sm = nb;
+  *max_ctas = nb * sms;
   *smem_bytes = smem;
   return cudaSuccess;
 }
 
 cudaError_t launch_scheduler(int path, const SchedParams& p, int grid, size_t smem, cudaStream_t stream) {
   if (path == kPathSplit3) {
-    sched_fused_kernel<<<grid, kFzThreads, smem, stream>>>(p);
-  } else if (path == kPathSplit3Wide) {
-    sched_wide_kernel<<<grid, kFzThreads, smem, stream>>>(p);
-  } else if (path == kPathSplit3Tma) {
-    sched_tma_kernel<<<grid, kTmThreads, smem, stream>>>(p);
+    sched_pair_kernel<<<grid, kPrThreads, smem, stream>>>(p);
   } else {
-    sched_fma_kernel<<<grid, kThreads, smem, stream>>>(p);
+    sched_fma_kernel<<<grid, kFmaThreads, smem, stream>>>(p);
   }
   return cudaGetLastError();
 }
