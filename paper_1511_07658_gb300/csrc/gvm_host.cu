@@ -138,12 +138,15 @@ struct gvm_ctx {
   std::atomic<int> ipc_servers{0};  // gvm_ipc servers using this manager
   int device = 0;
   std::vector<cudaStream_t> owned_streams;  // created by gvm_init, destroyed by gvm_shutdown
+  WorkerPool* workers = worker_pool_create();
   ~gvm_ctx() {
+    worker_pool_destroy(workers);
     for (cudaStream_t st : owned_streams) cudaStreamDestroy(st);
   }
 };
 
 namespace gvm {
+WorkerPool* ctx_workers(gvm_ctx* ctx) { return ctx->workers; }
 int ctx_mode(const gvm_ctx* ctx) { return ctx->cfg.mode; }
 int ctx_max_ranks(const gvm_ctx* ctx) { return ctx->cfg.max_ranks; }
 void ctx_servers_add(gvm_ctx* ctx, int delta) { ctx->ipc_servers.fetch_add(delta, std::memory_order_acq_rel); }

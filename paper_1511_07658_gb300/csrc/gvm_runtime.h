@@ -37,6 +37,13 @@ uint32_t encode_pair_maps(const float* A, const float* B, int32_t m, int64_t n, 
 cudaError_t scheduler_setup(int path, int sms, int* max_ctas, size_t* smem_bytes);
 cudaError_t launch_scheduler(int path, const SchedParams& p, int grid, size_t smem, cudaStream_t stream);
 
+// A manager's worker threads for the SPMD harnesses (gvm_spmd.cu): none until a
+// run needs them, then kept for the next run and joined with the manager.
+class WorkerPool;
+WorkerPool* worker_pool_create();
+void worker_pool_destroy(WorkerPool* pool);
+WorkerPool* ctx_workers(gvm_ctx* ctx);
+
 // Configuration of a manager, for the library's other host modules.
 int ctx_mode(const gvm_ctx* ctx);
 int ctx_max_ranks(const gvm_ctx* ctx);
