@@ -117,25 +117,38 @@ __device__ __forceinline__ uint32_t pub_check(uint32_t base, uint32_t seq, uint3
   return base ^ (seq * 0x9e3779b9u) ^ (task << 16) ^ cnt;
 }
 
-// One warp copies, for each of n tasks, `pieces` (8 or 16) 16-byte pieces
-// starting `at` bytes into its descriptor from the host ring to the device
-// table, kBatch reads of host memory in flight a lane.
-template <uint32_t kPieces, uint32_t kBatch>
-__device__ __forceinline__ void copy_bodies(const SchedParams& p, const uint32_t* list, uint32_t n, uint32_t at) {
-  const uint32_t lane = threadIdx.x & 31, total = n * kPieces;
+// One warp copies descriptors from the host ring to the device table: the
+// fields (8 pieces of 16 bytes) of the nf tasks in `fields`, the maps (16 pieces)
+// of the nm tasks in `maps`, kBatch reads of host memory in flight a lane (a
+// round trip takes 3 us).
+template <uint32_t kBatch>
+__device__ __forceinline__ void copy_bodies(const SchedParams& p, const uint32_t* fields, uint32_t nf,
+                                            const uint32_t* maps, uint32_t nm) {
+  const uint32_t lane = threadIdx.x & 31, split = nf * 8, total = split + nm * 16;
+  auto place = [&](uint32_t u, uint32_t& idx, uint32_t& at) {
+    const bool f = u < split;
+    const uint32_t w = u - split;
+    idx = f ? fields[u / 8] : maps[w / 16];
+    at = f ? kFieldsAt + 16 * (u % 8) : 16 * (w % 16);
+  };
 #pragma unroll 1
   for (uint32_t u0 = lane; u0 < total; u0 += 32 * kBatch) {
     uint4 v[kBatch];
 #pragma unroll
     for (uint32_t j = 0; j < kBatch; ++j) {
-      const uint32_t u = u0 + 32 * j;
-      if (u < total)
-        v[j] = ld_volatile_v4(reinterpret_cast<const uint8_t*>(&p.host_desc[list[u / kPieces]]) + at + 16 * (u % kPieces));
+      uint32_t idx, at;
+      if (u0 + 32 * j < total) {
+        place(u0 + 32 * j, idx, at);
+        v[j] = ld_volatile_v4(reinterpret_cast<const uint8_t*>(&p.host_desc[idx]) + at);
+      }
     }
 #pragma unroll
     for (uint32_t j = 0; j < kBatch; ++j) {
-      const uint32_t u = u0 + 32 * j;
-      if (u < total) st_cg_v4(reinterpret_cast<uint8_t*>(&p.tasks[list[u / kPieces]].body) + at + 16 * (u % kPieces), v[j]);
+      uint32_t idx, at;
+      if (u0 + 32 * j < total) {
+        place(u0 + 32 * j, idx, at);
+        st_cg_v4(reinterpret_cast<uint8_t*>(&p.tasks[idx].body) + at, v[j]);
+      }
     }
   }
 }
@@ -195,11 +208,10 @@ __device__ __forceinline__ IngestOut ingest_pass(const SchedParams& p, uint64_t*
     const uint32_t lanes = min(32u, p.ranks - g);
     if (lanes * quantum > space) quantum = space / lanes;
 
-    uint32_t r = 0, t = 0, take = 0, avail = 0;
-    uint32_t tidx[kMaxQuantum], tcnt[kMaxQuantum];
+    uint32_t r = 0, t = 0, take = 0, avail = 0, lim = 0;
+    uint32_t tcnt[kMaxQuantum];  // tiles of the taken tasks (0: nothing to publish); indexed statically
     uint32_t entries = 0, tiles = 0, maps = 0;  // maps: bit i = task i has tensor maps to copy
     const bool valid = (g + lane) < p.ranks;
-    uint32_t lim = 0;
     if (valid) {
       r = (rr + g + lane) % p.ranks;
       const uint32_t h = ld_acquire_sys(&p.host_heads[r].head);
@@ -208,8 +220,13 @@ __device__ __forceinline__ IngestOut ingest_pass(const SchedParams& p, uint64_t*
       lim = min(avail, quantum);
     }
     bool more = valid;
-#pragma unroll 1
-    for (uint32_t base = 0; base < kMaxQuantum && __any_sync(0xffffffffu, more && base < lim); base += kBatch) {
+#pragma unroll
+    for (uint32_t base = 0; base < kMaxQuantum; base += kBatch) {
+      if (!__any_sync(0xffffffffu, more && base < lim)) {
+#pragma unroll
+        for (uint32_t i = 0; i < kBatch; ++i) tcnt[base + i] = 0;
+        continue;
+      }
       uint4 h0[kBatch], h1[kBatch];
       uint32_t rdy[kBatch];
 #pragma unroll
@@ -224,6 +241,7 @@ __device__ __forceinline__ IngestOut ingest_pass(const SchedParams& p, uint64_t*
       }
 #pragma unroll
       for (uint32_t i = 0; i < kBatch; ++i) {
+        tcnt[base + i] = 0;
         if (more && base + i < lim) {
           const uint32_t s = t + base + i;
           const uint32_t idx = r * p.depth + (s & (p.depth - 1));
@@ -231,8 +249,7 @@ __device__ __forceinline__ IngestOut ingest_pass(const SchedParams& p, uint64_t*
           if ((flags & kFlagNeedsReady) && rdy[i] != s + 1u) {
             more = false;
           } else {
-            tidx[take] = idx;
-            tcnt[take] = 0;
+            ++take;
             if (tag != s + 1u) {
               bad = true;
             } else {
@@ -243,13 +260,12 @@ __device__ __forceinline__ IngestOut ingest_pass(const SchedParams& p, uint64_t*
                 __threadfence();
                 complete_task(p, idx, tag, flags, now);
               } else {
-                if (flags & (kFlagTmA | kFlagTmB)) maps |= 1u << take;
-                tcnt[take] = ntiles;
+                if (flags & (kFlagTmA | kFlagTmB)) maps |= 1u << (base + i);
+                tcnt[base + i] = ntiles;
                 ++entries;
                 tiles += ntiles;
               }
             }
-            ++take;
           }
         }
       }
@@ -258,25 +274,27 @@ __device__ __forceinline__ IngestOut ingest_pass(const SchedParams& p, uint64_t*
     // read relaxed: order the copies' data before what is published below.
     __threadfence();
 
-    // Copy the taken tasks' fields and maps.
-    const uint32_t nt = entries, ie = warp_incl_scan(nt), it = warp_incl_scan(tiles);
-    const uint32_t nm = (uint32_t)__popc(maps), im = warp_incl_scan(nm);
+    // Queue entries, and the lists of what to copy.
+    const uint32_t nm = (uint32_t)__popc(maps);
+    const uint32_t ie = warp_incl_scan(entries), it = warp_incl_scan(tiles), im = warp_incl_scan(nm);
     const uint32_t te = __shfl_sync(0xffffffffu, ie, 31), tt = __shfl_sync(0xffffffffu, it, 31);
     const uint32_t tm = __shfl_sync(0xffffffffu, im, 31);
-    uint64_t e0 = pub + ie - nt, b0 = ptiles + it - tiles;
-    uint32_t at = ie - nt, at_m = im - nm;
-    for (uint32_t i = 0; i < take; ++i) {
+    uint64_t e0 = pub + ie - entries, b0 = ptiles + it - tiles;
+    uint32_t at = ie - entries, at_m = im - nm;
+#pragma unroll
+    for (uint32_t i = 0; i < kMaxQuantum; ++i) {
       if (!tcnt[i]) continue;
-      list[at++] = tidx[i];
-      if ((maps >> i) & 1u) maps_list[at_m++] = tidx[i];
-      PubEntry e{b0, e0, tidx[i], 0, tcnt[i], pub_check((uint32_t)b0, (uint32_t)e0, tidx[i], tcnt[i])};
-      p.pubq[e0 & (p.qcap - 1)] = e;
+      const uint32_t idx = r * p.depth + ((t + i) & (p.depth - 1));
+      list[at++] = idx;
+      if ((maps >> i) & 1u) maps_list[at_m++] = idx;
+      uint4* pe = reinterpret_cast<uint4*>(&p.pubq[e0 & (p.qcap - 1)]);
+      st_cg_v4(pe, make_uint4((uint32_t)b0, (uint32_t)(b0 >> 32), (uint32_t)e0, (uint32_t)(e0 >> 32)));
+      st_cg_v4(pe + 1, make_uint4(idx, 0, tcnt[i], pub_check((uint32_t)b0, (uint32_t)e0, idx, tcnt[i])));
       ++e0;
       b0 += tcnt[i];
     }
     __syncwarp();
-    copy_bodies<8, 2 * kBatch>(p, list, te, kFieldsAt);
-    copy_bodies<16, 2 * kBatch>(p, maps_list, tm, 0);
+    copy_bodies<4 * kBatch>(p, list, te, maps_list, tm);
     __syncwarp();
     if (valid && take > 0) *reinterpret_cast<volatile uint32_t*>(&p.tail[r]) = t + take;
     pending += avail - take;
@@ -294,13 +312,12 @@ __device__ __forceinline__ IngestOut ingest_pass(const SchedParams& p, uint64_t*
       *reinterpret_cast<volatile uint64_t*>(&p.ctrl->quiet_until) = now + kQuietNs;
       if (p.drain) st_release_gpu(&p.ctrl->drained, 1u);  // under the lock: no later pass publishes
     }
+    *reinterpret_cast<volatile uint32_t*>(&p.ctrl->rr) = (rr + 1) % p.ranks;
     if (pub != pub0) {
-      st_release_gpu64(&p.ctrl->published, pub);
+      *reinterpret_cast<volatile uint64_t*>(&p.ctrl->published) = pub;
       st_release_gpu64(&p.ctrl->published_tiles, ptiles);
     }
-    *reinterpret_cast<volatile uint32_t*>(&p.ctrl->rr) = (rr + 1) % p.ranks;
-    __threadfence();
-    atomicExch(&p.ctrl->ingest_lock, 0u);
+    st_release_gpu(&p.ctrl->ingest_lock, 0u);
     if (any_bad) report_error(p, kStatusBadTask, 0, 0);
   }
   __syncwarp();
