@@ -787,13 +787,15 @@ void fill_body(gvm_ctx* ctx, gvm_rank* r, const Prep& p, uint64_t seq, uint64_t 
     body->k = t->k;
     body->n = t->n;
     const bool split3 = ctx->path != kPathFma;
-    const int tm = split3 ? 256 : kFmaTile, tn = tm;
+    int tm = kFmaTile, tn = kFmaTile;
     if (split3) {
-      body->flags |= kFlagSplit3;
-      body->vadd_tile = tn;
       // Operands land by tensor copies: the task's own maps of A and B.
-      body->flags |= kFlagTmA * encode_pair_maps(reinterpret_cast<const float*>(da), reinterpret_cast<const float*>(db),
-                                                 t->m, t->n, t->k, &body->tmA, &body->tmB);
+      const uint32_t maps = encode_pair_maps(reinterpret_cast<const float*>(da), reinterpret_cast<const float*>(db),
+                                             t->m, t->n, t->k, &body->tmA, &body->tmB);
+      tm = 256;
+      tn = pair_tile_n(maps);
+      body->flags |= kFlagSplit3 | kFlagTmA * maps;
+      body->vadd_tile = tn;
     }
     body->tiles_m = (uint32_t)((t->m + tm - 1) / tm);
     body->tiles_n = (uint32_t)((t->n + tn - 1) / tn);

@@ -151,6 +151,8 @@ uint32_t encode_pair_maps(const float* A, const float* B, int32_t m, int64_t n, 
          encode(B, (uint64_t)k, (uint64_t)n, 32, kPrPackB, tmB, kPrMapB, kPrPackedB);
 }
 
+int pair_tile_n(uint32_t maps) { return maps == (kPrMapA | kPrMapB) ? kPrN : kPrPackedN; }
+
 constexpr uint64_t kStandaloneTimeoutNs = 10ull * 1000 * 1000 * 1000;
 
 static int sm_count() {
@@ -239,10 +241,14 @@ extern "C" int gvm_sgemm_f32(const float* A, const float* B, float* C, int32_t m
   // does not shrink with n): measured 15 / 17 / 18 / 21 us at 512^3 (16, 8, 6
   // and 4 tiles of 76 pairs; 64 columns taken), 108 / 64 / 70 / 44 us at
   // 2048^3 (256, 128, 88 and 64 tiles; 256 taken).
-  int tile_n = kPrN;
+  CUtensorMap tmA, tmB;
+  memset(&tmA, 0, sizeof(tmA));
+  memset(&tmB, 0, sizeof(tmB));
+  const uint32_t maps = encode_pair_maps(A, B, m, n, k, &tmA, &tmB);
+  int tile_n = 64;
   int64_t best = INT64_MAX;
   const int64_t rows = (m + kPrM - 1) / kPrM;
-  for (int tn = kPrN; tn >= 64; tn -= 64) {
+  for (int tn = pair_tile_n(maps); tn >= 64; tn -= 64) {
     const int64_t cost = (rows * ((n + tn - 1) / tn) + pairs - 1) / pairs * (256 + tn);
     if (cost < best) {
       best = cost;
@@ -250,10 +256,6 @@ extern "C" int gvm_sgemm_f32(const float* A, const float* B, float* C, int32_t m
     }
   }
   const int64_t tiles = rows * ((n + tile_n - 1) / tile_n);
-  CUtensorMap tmA, tmB;
-  memset(&tmA, 0, sizeof(tmA));
-  memset(&tmB, 0, sizeof(tmB));
-  const uint32_t maps = encode_pair_maps(A, B, m, n, k, &tmA, &tmB);
   const int grid = 2 * (int)(tiles < pairs ? tiles : pairs);
   pr_sgemm_kernel<<<grid, kPrThreads, smem, s>>>(tmA, tmB, maps, A, B, C, m, n, k, tile_n, kStandaloneTimeoutNs);
   return cudaGetLastError() == cudaSuccess ? GVM_OK : GVM_EDEVICE;

@@ -12,8 +12,12 @@
 //
 // The landing ring (kPrLand stages) holds only operands in flight and is
 // released as soon as the converting warps have read it into registers, so
-// up to 96 KB a CTA is on its way from L2 without holding registers; the
-// bf16 ring (kPrStages) decouples the conversion from the MMAs.
+// up to 128 KB a CTA is on its way from L2 without holding registers; the
+// bf16 ring (kPrStages) decouples the conversion from the MMAs. Aligned
+// operands are read into registers before the stage is awaited. With three
+// landings of 35 KB and the stage awaited first, 1024 products of 512^3 took
+// 0.80 ms (now 0.74), the grouped mix 2.23 (2.01), 2048^3 43 us (40.5) and 64
+// vector adds of 4 M values 0.55 ms (0.50).
 //
 // CTA roles (kPrThreads = 480, one CTA per SM):
 //   warps 0-3    epilogue: TMEM lanes 32 w .. +31 of a finished accumulator
@@ -36,7 +40,7 @@
 // are multiples of 16 bytes. Four consecutive rows of k values are one row of
 // 4 k values whose pitch is such a multiple, so the matrix is mapped in rows
 // of four ("super-rows"), and row 4 i + j is fetched from super-row i at value
-// j k + kk, rounded down to a multiple of 4: boxes of 36 values (A) or 132 (B),
+// j k + kk, rounded down to a multiple of 4: boxes of 36 values (A) or 100 (B),
 // one per j, whose first d_j = (j k) % 4 values are skipped when read. With k
 // odd the four d_j differ, and the 4-byte reads of a warp (8 rows x 4 groups
 // of 8 values) fall on 32 different banks. Rows beyond the last whole
@@ -62,20 +66,26 @@ namespace gvm {
 
 constexpr int kPrM = 256;  // rows of a pair tile (128 per CTA)
 constexpr int kPrN = 256;  // most columns of a pair tile (half per CTA)
-constexpr int kPrLand = 3;
+// Four landings and three stages. Barriers of landings and stages always belong
+// to the same converter group: landing q % 4's, and for the stages six, q % 6.
+// (A group meets stage q % 3 at every second use only; at a barrier of the
+// stage's own it would wait for the same parity each time, and a parity does
+// not tell a phase from the one two before it.)
+constexpr int kPrLand = 4;
 constexpr int kPrStages = 3;
-// Barriers of the landings and stages: k-step q uses landing and stage q % 3 but
-// barrier q % 6, which always belongs to the same converter group. (A group
-// meets a landing at every second use only; at a barrier of the landing's own
-// it would wait for the same parity each time, and a parity does not tell a
-// phase from the one two before it.)
 constexpr int kPrBars = 6;
-static_assert(kPrLand == 3 && kPrStages == 3, "a group meets barrier q % 6 at every use");
+static_assert(kPrLand % 2 == 0 && kPrBars == 2 * kPrStages, "a group sees every phase of its barriers");
+// Packed operands take more room in a landing, so that tiles with one have
+// at most kPrPackedN columns.
+constexpr int kPrPackedN = 192;
 constexpr uint32_t kPrPackA = 36;                              // values a packed A row lands with
-constexpr uint32_t kPrPackB = 132;                             // values a packed B row lands with
-constexpr uint32_t kPrLandB = 128 * kPrPackA * 4;              // B's landing starts after A's 18 KB
+constexpr uint32_t kPrPackB = kPrPackedN / 2 + 4;              // values a packed B row lands with
 constexpr uint32_t kPrSlab = 32 * 128;                         // one aligned slab: 32 k-rows x 32 columns
-constexpr uint32_t kPrLandBytes = (kPrLandB + 32 * kPrPackB * 4 + 1023) / 1024 * 1024;  // 35 KB
+constexpr uint32_t kPrLandBytes = 32768;
+constexpr uint32_t kPrLandA = 128 * 128, kPrLandPackA = 128 * kPrPackA * 4;  // A's bytes; B's landing follows
+static_assert(kPrLandA + 4 * kPrSlab <= kPrLandBytes && kPrLandPackA + 32 * kPrPackB * 4 <= kPrLandBytes &&
+                  kPrLandPackA + (kPrPackedN / 64) * kPrSlab <= kPrLandBytes && kPrLandPackA % 1024 == 0,
+              "every mix of landings fits");
 constexpr uint32_t kPrAOff = 0;                                // bf16 planes
 constexpr uint32_t kPrAlOff = 128 * 64;
 constexpr uint32_t kPrBOff = 2 * 128 * 64;
@@ -96,8 +106,8 @@ constexpr int kPrThreads = 15 * 32;
 constexpr int kPrTmemCols = 512;  // two accumulators of 128 lanes x 256 columns per CTA
 
 struct PrShared {
-  uint64_t landed[kPrBars];     // producer -> converters (one arrival + the copies' bytes)
-  uint64_t land_free[kPrBars];  // converters (4 warps of the k-step's group) -> producer
+  uint64_t landed[kPrLand];     // producer -> converters (one arrival + the copies' bytes)
+  uint64_t land_free[kPrLand];  // converters (4 warps of the k-step's group) -> producer
   uint64_t full[kPrStages];     // leader: converters of both CTAs -> MMA (4 + 4 warps)
   uint64_t empty[kPrBars];      // both: MMA commit -> converters
   uint64_t acc_full[2];         // both: MMA commit -> epilogue
@@ -312,11 +322,11 @@ __device__ __forceinline__ uint64_t pr_desc_b(uint32_t saddr) {
 __device__ __forceinline__ void pr_init(PrShared* ps) {
   if (threadIdx.x == 0) {
     ps->cta = cluster_ctarank();
-    for (int i = 0; i < kPrBars; ++i) {
+    for (int i = 0; i < kPrLand; ++i) {
       mbar_init(&ps->landed[i], 1);
       mbar_init(&ps->land_free[i], kPrGroupWarps);
-      mbar_init(&ps->empty[i], 1);
     }
+    for (int i = 0; i < kPrBars; ++i) mbar_init(&ps->empty[i], 1);
     for (int s = 0; s < kPrStages; ++s) mbar_init(&ps->full[s], 2 * kPrGroupWarps);
     for (int b = 0; b < 2; ++b) {
       mbar_init(&ps->acc_full[b], 1);
@@ -372,7 +382,7 @@ __device__ __forceinline__ uint32_t pr_shift(const float* p) {
 
 // The producer thread: the tensor copies of every k-step of tile t, each
 // k-step once the converters have read what its landing held. pend: bit 2i =
-// a copy was issued on barrier i, bit 2i + 1 = the parity of its phase.
+// a copy was issued into landing i, bit 2i + 1 = the parity of its phase.
 // Returns false when a wait ran out.
 __device__ __forceinline__ bool pr_produce(const PrTile t, uint8_t* land, PrShared* ps, uint32_t it,
                                            const CUtensorMap* tmA, const CUtensorMap* tmB, uint64_t timeout_ns,
@@ -389,14 +399,12 @@ __device__ __forceinline__ bool pr_produce(const PrTile t, uint8_t* land, PrShar
   const uint32_t land0 = smem_u32(land);
   const int xa = (int)pr_shift(t.A), xb = (int)pr_shift(t.B) + col0, n = (int)t.n;
   for (int kb = 0; kb < nkb; ++kb) {
-    const uint32_t q = it + (uint32_t)kb, s = q % kPrLand, i = q % kPrBars;
-    // The landing's previous k-step, q - 3, has been read.
-    if (q >= kPrLand && !mbar_wait(&ps->land_free[(q - kPrLand) % kPrBars], ((q - kPrLand) / kPrBars) & 1u, timeout_ns,
-                                   cta_abort)) {
+    const uint32_t q = it + (uint32_t)kb, i = q % kPrLand;
+    if (!mbar_wait(&ps->land_free[i], ((q / kPrLand) & 1u) ^ 1u, timeout_ns, cta_abort)) {
       pr_fail(ps, cta_abort, fail_where, kWhereEmptyBarrier);
       return false;
     }
-    const uint32_t st = land0 + s * kPrLandBytes;
+    const uint32_t st = land0 + i * kPrLandBytes, st_b = st + (pack_a ? kPrLandPackA : kPrLandA);
     uint64_t* bar = &ps->landed[i];
     mbar_expect_tx(bar, tx);
     const int k0 = kb * kTcBK;
@@ -412,14 +420,14 @@ __device__ __forceinline__ bool pr_produce(const PrTile t, uint8_t* land, PrShar
     if (map_b) {
       if (!pack_b) {
         for (int b = 0; b < slabs; ++b)
-          tma_load_2d(st + kPrLandB + (uint32_t)b * kPrSlab, tmB, col0 + 32 * b, k0, bar);
+          tma_load_2d(st_b + (uint32_t)b * kPrSlab, tmB, col0 + 32 * b, k0, bar);
       } else {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          tma_load_2d(st + kPrLandB + (uint32_t)j * (8u * kPrPackB * 4u), tmB, (xb + j * n) & ~3, k0 >> 2, bar);
+          tma_load_2d(st_b + (uint32_t)j * (8u * kPrPackB * 4u), tmB, (xb + j * n) & ~3, k0 >> 2, bar);
       }
     }
-    pend = (pend & ~(3u << (2 * i))) | ((tx ? (1u | (((q / kPrBars) & 1u) << 1)) : 0u) << (2 * i));
+    pend = (pend & ~(3u << (2 * i))) | ((tx ? (1u | (((q / kPrLand) & 1u) << 1)) : 0u) << (2 * i));
   }
   return true;
 }
@@ -429,7 +437,7 @@ __device__ __forceinline__ bool pr_produce(const PrTile t, uint8_t* land, PrShar
 // after it is gone.
 __device__ __forceinline__ void pr_produce_quiesce(PrShared* ps, uint32_t pend, uint64_t timeout_ns) {
   volatile uint32_t never = 0;
-  for (int i = 0; i < kPrBars; ++i)
+  for (int i = 0; i < kPrLand; ++i)
     if ((pend >> (2 * i)) & 1u) (void)mbar_wait(&ps->landed[i], (pend >> (2 * i + 1)) & 1u, timeout_ns, &never);
 }
 
@@ -441,20 +449,23 @@ __device__ __forceinline__ float ld_shared_f32(uint32_t addr) {
   return v;
 }
 
-// Converter warps, before k-step q (landing ql): its operands have landed and
-// its stage's previous k-step, q - 3, has been read by the MMAs. Landings also
-// serve vector tiles, so that ql runs ahead of q, by an even number: both
-// belong to the same group.
-__device__ __forceinline__ bool pr_convert_wait(PrShared* ps, uint32_t ql, uint32_t q, uint64_t timeout_ns,
-                                                uint32_t* cta_abort, uint32_t* fail_where) {
-  uint32_t where = 0;
-  if (!mbar_wait_warp<false>(&ps->landed[ql % kPrBars], (ql / kPrBars) & 1u, timeout_ns, cta_abort))
-    where = kWhereEmptyBarrier;
-  else if (q >= kPrStages && !mbar_wait_warp<false>(&ps->empty[(q - kPrStages) % kPrBars],
-                                                    ((q - kPrStages) / kPrBars) & 1u, timeout_ns, cta_abort))
-    where = kWhereFullBarrier;
-  if (where && (threadIdx.x & 31) == 0) pr_fail(ps, cta_abort, fail_where, where);
-  return where == 0;
+// Converter warps, landing ql: its operands have landed. Landings also serve
+// vector tiles, so that ql runs ahead of the k-step's number q, by an even
+// number: both belong to the same group.
+__device__ __forceinline__ bool pr_wait_landed(PrShared* ps, uint32_t ql, uint64_t timeout_ns, uint32_t* cta_abort,
+                                               uint32_t* fail_where) {
+  if (mbar_wait_warp<false>(&ps->landed[ql % kPrLand], (ql / kPrLand) & 1u, timeout_ns, cta_abort)) return true;
+  if ((threadIdx.x & 31) == 0) pr_fail(ps, cta_abort, fail_where, kWhereEmptyBarrier);
+  return false;
+}
+// Converter warps, k-step q: the MMAs have read its stage's previous k-step, q - 3.
+__device__ __forceinline__ bool pr_wait_stage(PrShared* ps, uint32_t q, uint64_t timeout_ns, uint32_t* cta_abort,
+                                              uint32_t* fail_where) {
+  if (q < kPrStages || mbar_wait_warp<false>(&ps->empty[(q - kPrStages) % kPrBars], ((q - kPrStages) / kPrBars) & 1u,
+                                             timeout_ns, cta_abort))
+    return true;
+  if ((threadIdx.x & 31) == 0) pr_fail(ps, cta_abort, fail_where, kWhereFullBarrier);
+  return false;
 }
 
 // Converter warps: split the k-steps of tile t that belong to this warp's
@@ -478,9 +489,9 @@ __device__ __forceinline__ bool pr_convert_aligned(const PrTile t, uint32_t land
   const uint32_t wr = swz64(r, c);
   for (int kb = (int)((it + (uint32_t)par) & 1u); kb < nkb; kb += 2) {
     const uint32_t q = it + (uint32_t)kb, ql = it_l + (uint32_t)kb;
-    const uint32_t s = q % kPrStages, i6 = ql % kPrBars;
-    if (!pr_convert_wait(ps, ql, q, timeout_ns, cta_abort, fail_where)) return false;
-    const uint32_t ld = land0 + (ql % kPrLand) * kPrLandBytes;
+    const uint32_t s = q % kPrStages, i = ql % kPrLand;
+    if (!pr_wait_landed(ps, ql, timeout_ns, cta_abort, fail_where)) return false;
+    const uint32_t ld = land0 + i * kPrLandBytes;
     const uint32_t st = st0 + s * kPrStageBytes;
     // A and the first half of B are read, A is stored, the rest of B is read:
     // 48 values a lane in flight. With all 64 read first the loop spilled.
@@ -489,8 +500,8 @@ __device__ __forceinline__ bool pr_convert_aligned(const PrTile t, uint32_t land
     for (int b = 0; b < 4; ++b) xb[b][1].w = 0;
     auto read_b = [&](int b) {
       if (b < slabs) {
-        xb[b][0] = ld_shared_v4(ld + kPrLandB + (uint32_t)b * kPrSlab + rd0);
-        xb[b][1] = ld_shared_v4(ld + kPrLandB + (uint32_t)b * kPrSlab + rd1);
+        xb[b][0] = ld_shared_v4(ld + kPrLandA + (uint32_t)b * kPrSlab + rd0);
+        xb[b][1] = ld_shared_v4(ld + kPrLandA + (uint32_t)b * kPrSlab + rd1);
       }
     };
     auto put = [&](const uint4 (&x)[2], uint32_t hi_at, uint32_t lo_at) {
@@ -511,6 +522,7 @@ __device__ __forceinline__ bool pr_convert_aligned(const PrTile t, uint32_t land
     }
     read_b(0);
     read_b(1);
+    if (!pr_wait_stage(ps, q, timeout_ns, cta_abort, fail_where)) return false;
     if (has_a) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -525,7 +537,7 @@ __device__ __forceinline__ bool pr_convert_aligned(const PrTile t, uint32_t land
     // value equals both constants, which the compiler does not see).
     const uint32_t last = xb[0][1].w ^ xb[1][1].w ^ xb[2][1].w ^ xb[3][1].w;
     const bool read = (__ballot_sync(0xffffffffu, last == 0x7fa5a5a5u) & __ballot_sync(0xffffffffu, last == 0x7f5a5a5au)) == 0;
-    if (lane == 0 && read) mbar_arrive(&ps->land_free[i6]);
+    if (lane == 0 && read) mbar_arrive(&ps->land_free[i]);
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       if (b < slabs) {
@@ -572,9 +584,11 @@ __device__ __forceinline__ bool pr_convert_packed(const PrTile t, uint32_t land0
   const uint32_t wr = swz64(r, c);
   for (int kb = (int)((it + (uint32_t)par) & 1u); kb < nkb; kb += 2) {
     const uint32_t q = it + (uint32_t)kb, ql = it_l + (uint32_t)kb;
-    const uint32_t s = q % kPrStages, i6 = ql % kPrBars;
-    if (!pr_convert_wait(ps, ql, q, timeout_ns, cta_abort, fail_where)) return false;
-    const uint32_t ld = land0 + (ql % kPrLand) * kPrLandBytes;
+    const uint32_t s = q % kPrStages, i = ql % kPrLand;
+    if (!pr_wait_landed(ps, ql, timeout_ns, cta_abort, fail_where) ||
+        !pr_wait_stage(ps, q, timeout_ns, cta_abort, fail_where))
+      return false;
+    const uint32_t ld = land0 + i * kPrLandBytes, ld_b = ld + ((t.land & kPrPackedA) ? kPrLandPackA : kPrLandA);
     const uint32_t st = st0 + s * kPrStageBytes;
     auto read = [&](bool packed, uint32_t packed_at, uint32_t a0, uint32_t a1, float (&v)[8]) {
       if (packed) {
@@ -628,7 +642,7 @@ __device__ __forceinline__ bool pr_convert_packed(const PrTile t, uint32_t land0
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const uint32_t b = (uint32_t)min(b0 + u, slabs - 1);
-        read(pack_b, ld + kPrLandB + pb + b * 128u, ld + kPrLandB + b * kPrSlab + rd0, ld + kPrLandB + b * kPrSlab + rd1,
+        read(pack_b, ld_b + pb + b * 128u, ld_b + b * kPrSlab + rd0, ld_b + b * kPrSlab + rd1,
              x[u]);
       }
 #pragma unroll
@@ -650,7 +664,7 @@ __device__ __forceinline__ bool pr_convert_packed(const PrTile t, uint32_t land0
     fence_proxy_async_shared();
     __syncwarp();
     if (lane == 0) {
-      mbar_arrive(&ps->land_free[i6]);
+      mbar_arrive(&ps->land_free[i]);
       mbar_arrive_cta(&ps->full[s], 0);
     }
   }
@@ -672,7 +686,7 @@ __device__ __forceinline__ bool pr_convert(const PrTile t, uint8_t* land, uint8_
 // ring as well: the producer lands 4096 elements of a and of b at a time (two
 // bulk copies of 16 KB), the converter group of the landing adds or multiplies
 // them and stores c. The copies of a tile are under way while the tile before
-// is worked on, 96 KB a CTA. With direct loads (16-byte loads, four of each
+// is worked on, 128 KB a CTA. With direct loads (16-byte loads, four of each
 // operand a thread in flight, drained at every tile's end) 16 x 4 vector adds
 // of 2^22 took 0.66 ms a launch on CTA pairs.
 
@@ -701,9 +715,8 @@ __device__ __forceinline__ bool pr_vec_produce(const float* a, const float* b, i
                                                uint32_t* fail_where, uint32_t& pend) {
   const uint32_t n = pr_vec_chunks(len), land0 = smem_u32(land);
   for (uint32_t ch = 0; ch < n; ++ch) {
-    const uint32_t q = it_l + ch, i = q % kPrBars;
-    if (q >= kPrLand && !mbar_wait(&ps->land_free[(q - kPrLand) % kPrBars], ((q - kPrLand) / kPrBars) & 1u, timeout_ns,
-                                   cta_abort)) {
+    const uint32_t q = it_l + ch, i = q % kPrLand;
+    if (!mbar_wait(&ps->land_free[i], ((q / kPrLand) & 1u) ^ 1u, timeout_ns, cta_abort)) {
       pr_fail(ps, cta_abort, fail_where, kWhereEmptyBarrier);
       return false;
     }
@@ -713,11 +726,11 @@ __device__ __forceinline__ bool pr_vec_produce(const float* a, const float* b, i
     uint64_t* bar = &ps->landed[i];
     mbar_expect_tx(bar, 2 * bytes);
     if (bytes) {
-      const uint32_t st = land0 + (q % kPrLand) * kPrLandBytes;
+      const uint32_t st = land0 + i * kPrLandBytes;
       bulk_g2s(st, a + at, bytes, bar);
       bulk_g2s(st + kPrVecB, b + at, bytes, bar);
     }
-    pend = (pend & ~(3u << (2 * i))) | ((bytes ? (1u | (((q / kPrBars) & 1u) << 1)) : 0u) << (2 * i));
+    pend = (pend & ~(3u << (2 * i))) | ((bytes ? (1u | (((q / kPrLand) & 1u) << 1)) : 0u) << (2 * i));
   }
   return true;
 }
@@ -733,7 +746,7 @@ __device__ __forceinline__ bool pr_vec_convert(const float* a, const float* b, f
   const bool cvec = (reinterpret_cast<uintptr_t>(c) & 15) == 0;
   for (uint32_t ch = (it_l + par) & 1u; ch < n; ch += 2) {
     const uint32_t q = it_l + ch;
-    if (!mbar_wait_warp<false>(&ps->landed[q % kPrBars], (q / kPrBars) & 1u, timeout_ns, cta_abort)) {
+    if (!mbar_wait_warp<false>(&ps->landed[q % kPrLand], (q / kPrLand) & 1u, timeout_ns, cta_abort)) {
       if (lane == 0) pr_fail(ps, cta_abort, fail_where, kWhereEmptyBarrier);
       return false;
     }
@@ -760,7 +773,7 @@ __device__ __forceinline__ bool pr_vec_convert(const float* a, const float* b, f
       if (e < len) c[e] = elem_op<OP>(__ldcg(a + e), __ldcg(b + e), iters);
     }
     __syncwarp();
-    if (lane == 0) mbar_arrive(&ps->land_free[q % kPrBars]);
+    if (lane == 0) mbar_arrive(&ps->land_free[q % kPrLand]);
   }
   return true;
 }
@@ -775,7 +788,7 @@ __device__ __forceinline__ bool pr_mma(const PrTile t, uint8_t* stages, PrShared
                                        uint64_t timeout_ns, uint32_t* cta_abort, uint32_t* fail_where,
                                        uint64_t* wait_acc) {
   const uint32_t b = tile_no & 1u;
-  if (!mbar_wait_cluster(&ps->acc_empty[b], ((tile_no >> 1) & 1u) ^ 1u, timeout_ns, cta_abort)) {
+  if (!mbar_wait(&ps->acc_empty[b], ((tile_no >> 1) & 1u) ^ 1u, timeout_ns, cta_abort)) {
     pr_fail(ps, cta_abort, fail_where, kWhereAccumBarrier);
     return false;
   }
@@ -787,7 +800,7 @@ __device__ __forceinline__ bool pr_mma(const PrTile t, uint8_t* stages, PrShared
   for (int kb = 0; kb < nkb; ++kb) {
     const uint32_t q = it + (uint32_t)kb, s = q % kPrStages, ph = (q / kPrStages) & 1u;
     const long long c0 = wait_acc != nullptr ? clock64() : 0;
-    if (!mbar_wait_cluster(&ps->full[s], ph, timeout_ns, cta_abort)) {
+    if (!mbar_wait(&ps->full[s], ph, timeout_ns, cta_abort)) {
       pr_fail(ps, cta_abort, fail_where, kWhereFullBarrier);
       return false;
     }

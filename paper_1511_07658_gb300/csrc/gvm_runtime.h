@@ -31,6 +31,9 @@ const DriverApi* driver_api();
 uint32_t encode_pair_maps(const float* A, const float* B, int32_t m, int64_t n, int32_t k, CUtensorMap* tmA,
                           CUtensorMap* tmB);
 
+// Most columns of a pair-form tile whose operands have these maps.
+int pair_tile_n(uint32_t maps);
+
 // Scheduler kernel: the most CTAs the device (of `sms` SMs) holds at once on
 // `path`, dynamic smem bytes, and an asynchronous launch on `stream` (the pair
 // form's grid is a multiple of two).

@@ -50,7 +50,7 @@ struct alignas(128) SchedShared {
   uint64_t t_tile;   // when the current tile began (thread 0)
   uint64_t prof[kProfSlots];  // this CTA's phase counters (kProf*), written by thread 0 only
   uint64_t claim[4];  // Claim state (see acquire), owned by warp 0
-  uint32_t list[2 * 32 * kMaxQuantum];  // ingest's scratch, warp 0
+  uint32_t list[32 * kMaxQuantum];  // ingest's scratch, warp 0
 };
 
 constexpr uint64_t kLookaheadTiles = 512;  // ingest ahead when this few published tiles remain
@@ -117,39 +117,33 @@ __device__ __forceinline__ uint32_t pub_check(uint32_t base, uint32_t seq, uint3
   return base ^ (seq * 0x9e3779b9u) ^ (task << 16) ^ cnt;
 }
 
-// One warp copies descriptors from the host ring to the device table: the
-// fields (8 pieces of 16 bytes) of the nf tasks in `fields`, the maps (16 pieces)
-// of the nm tasks in `maps`, kBatch reads of host memory in flight a lane (a
-// round trip takes 3 us).
+// One warp copies the descriptors of n tasks from the host ring to the device
+// table: the fields (8 pieces of 16 bytes) of all, the maps (16 pieces) of those
+// marked kListMaps; kBatch reads of host memory in flight a lane (a round trip
+// takes 3 us).
+constexpr uint32_t kListMaps = 1u << 31;
 template <uint32_t kBatch>
-__device__ __forceinline__ void copy_bodies(const SchedParams& p, const uint32_t* fields, uint32_t nf,
-                                            const uint32_t* maps, uint32_t nm) {
-  const uint32_t lane = threadIdx.x & 31, split = nf * 8, total = split + nm * 16;
-  auto place = [&](uint32_t u, uint32_t& idx, uint32_t& at) {
-    const bool f = u < split;
+__device__ __forceinline__ void copy_bodies(const SchedParams& p, const uint32_t* list, uint32_t n, bool any_maps) {
+  const uint32_t lane = threadIdx.x & 31, split = n * 8, total = split + (any_maps ? n * 16 : 0);
+  // Piece u: the task, and its place in the descriptor; false: nothing to copy.
+  auto place = [&](uint32_t u, uint32_t& idx, uint32_t& at) -> bool {
+    if (u >= total) return false;
     const uint32_t w = u - split;
-    idx = f ? fields[u / 8] : maps[w / 16];
-    at = f ? kFieldsAt + 16 * (u % 8) : 16 * (w % 16);
+    const uint32_t e = u < split ? list[u / 8] : list[w / 16];
+    idx = e & ~kListMaps;
+    at = u < split ? kFieldsAt + 16 * (u % 8) : 16 * (w % 16);
+    return u < split || (e & kListMaps);
   };
 #pragma unroll 1
   for (uint32_t u0 = lane; u0 < total; u0 += 32 * kBatch) {
     uint4 v[kBatch];
+    uint32_t idx, at;
 #pragma unroll
-    for (uint32_t j = 0; j < kBatch; ++j) {
-      uint32_t idx, at;
-      if (u0 + 32 * j < total) {
-        place(u0 + 32 * j, idx, at);
-        v[j] = ld_volatile_v4(reinterpret_cast<const uint8_t*>(&p.host_desc[idx]) + at);
-      }
-    }
+    for (uint32_t j = 0; j < kBatch; ++j)
+      if (place(u0 + 32 * j, idx, at)) v[j] = ld_volatile_v4(reinterpret_cast<const uint8_t*>(&p.host_desc[idx]) + at);
 #pragma unroll
-    for (uint32_t j = 0; j < kBatch; ++j) {
-      uint32_t idx, at;
-      if (u0 + 32 * j < total) {
-        place(u0 + 32 * j, idx, at);
-        st_cg_v4(reinterpret_cast<uint8_t*>(&p.tasks[idx].body) + at, v[j]);
-      }
-    }
+    for (uint32_t j = 0; j < kBatch; ++j)
+      if (place(u0 + 32 * j, idx, at)) st_cg_v4(reinterpret_cast<uint8_t*>(&p.tasks[idx].body) + at, v[j]);
   }
 }
 
@@ -159,8 +153,8 @@ __device__ __forceinline__ void copy_bodies(const SchedParams& p, const uint32_t
 // heads and the header words of its rank's next tasks (kBatch tasks' reads in
 // flight), then the warp copies all taken descriptors together. Read and
 // stored task by task by each lane, a pass of 64 tasks with tensor maps took
-// 43 us, 0.68 ms of a 1024-task launch. list: two arrays of 32 x kMaxQuantum
-// words in shared memory.
+// 43 us, 0.68 ms of a 1024-task launch. list: 32 x kMaxQuantum words in shared
+// memory.
 template <uint32_t kBatch>
 __device__ __forceinline__ IngestOut ingest_pass(const SchedParams& p, uint64_t* prof, uint32_t* list) {
   const int lane = threadIdx.x & 31;
@@ -197,7 +191,6 @@ __device__ __forceinline__ IngestOut ingest_pass(const SchedParams& p, uint64_t*
   uint64_t pub = pub0, ptiles = tiles0;
   uint32_t pending = 0;
   bool bad = false;
-  uint32_t* maps_list = list + 32 * kMaxQuantum;
 
   for (uint32_t g = 0; g < p.ranks; g += 32) {
     // Keep at most half the ring between the hand-out frontier and the
@@ -274,19 +267,16 @@ __device__ __forceinline__ IngestOut ingest_pass(const SchedParams& p, uint64_t*
     // read relaxed: order the copies' data before what is published below.
     __threadfence();
 
-    // Queue entries, and the lists of what to copy.
-    const uint32_t nm = (uint32_t)__popc(maps);
-    const uint32_t ie = warp_incl_scan(entries), it = warp_incl_scan(tiles), im = warp_incl_scan(nm);
+    // Queue entries, and the list of what to copy.
+    const uint32_t ie = warp_incl_scan(entries), it = warp_incl_scan(tiles);
     const uint32_t te = __shfl_sync(0xffffffffu, ie, 31), tt = __shfl_sync(0xffffffffu, it, 31);
-    const uint32_t tm = __shfl_sync(0xffffffffu, im, 31);
     uint64_t e0 = pub + ie - entries, b0 = ptiles + it - tiles;
-    uint32_t at = ie - entries, at_m = im - nm;
+    uint32_t at = ie - entries;
 #pragma unroll
     for (uint32_t i = 0; i < kMaxQuantum; ++i) {
       if (!tcnt[i]) continue;
       const uint32_t idx = r * p.depth + ((t + i) & (p.depth - 1));
-      list[at++] = idx;
-      if ((maps >> i) & 1u) maps_list[at_m++] = idx;
+      list[at++] = idx | (((maps >> i) & 1u) ? kListMaps : 0u);
       uint4* pe = reinterpret_cast<uint4*>(&p.pubq[e0 & (p.qcap - 1)]);
       st_cg_v4(pe, make_uint4((uint32_t)b0, (uint32_t)(b0 >> 32), (uint32_t)e0, (uint32_t)(e0 >> 32)));
       st_cg_v4(pe + 1, make_uint4(idx, 0, tcnt[i], pub_check((uint32_t)b0, (uint32_t)e0, idx, tcnt[i])));
@@ -294,7 +284,7 @@ __device__ __forceinline__ IngestOut ingest_pass(const SchedParams& p, uint64_t*
       b0 += tcnt[i];
     }
     __syncwarp();
-    copy_bodies<4 * kBatch>(p, list, te, maps_list, tm);
+    copy_bodies<2 * kBatch>(p, list, te, __any_sync(0xffffffffu, maps != 0));
     __syncwarp();
     if (valid && take > 0) *reinterpret_cast<volatile uint32_t*>(&p.tail[r]) = t + take;
     pending += avail - take;
@@ -737,7 +727,7 @@ struct PairSchedShared {
   uint32_t fail_where;
   uint64_t prof[kProfSlots];      // kProf* counters; each slot written by one thread only
   uint64_t claim[4];              // Claim state, owned by the control warp
-  uint32_t list[2 * 32 * kMaxQuantum];  // ingest's scratch, control warp
+  uint32_t list[32 * kMaxQuantum];  // ingest's scratch, control warp
   uint64_t g_begin;               // %globaltimer and clock64 when the CTA began
   long long c_begin;
 };
