@@ -219,7 +219,12 @@ def peaks():
 
 # The sources the scheduler kernels are compiled from (host code does not
 # change their DRAM traffic per tile).
-KERNEL_SOURCES = ("gvm_sched.cu", "gvm_fused.cuh", "gvm_wide.cuh", "gvm_tma.cuh", "gvm_device.cuh", "gvm_internal.h")
+KERNEL_SOURCES = ("gvm_sched.cu", "gvm_pair.cuh", "gvm_device.cuh", "gvm_internal.h")
+
+
+def scheduler_kernel(path):
+    """The scheduler kernel that runs a manager of this SGEMM path."""
+    return "sched_fma_kernel" if path == "fma" else "sched_pair_kernel"
 
 
 def kernel_source_hash():
@@ -886,8 +891,7 @@ def gpu_arm(args, w, desc, rank, world):
         peak = pk["hbm_gbs"]
         roof = {"bound": "hbm", "unit": "GB/s", "peak_basis": f"HBM copy {pk['hbm_gbs']} GB/s ({pk_kind})"}
         achieved = byts / kmean / 1e9
-    kname = {"split3": "sched_fused_kernel", "split3_wide": "sched_wide_kernel",
-             "split3_tma": "sched_tma_kernel"}.get(args.path, "sched_fma_kernel")
+    kname = scheduler_kernel(args.path)
     key = f"{kname}/{args.workload}"
     roof.update({"kernel": f"gvm::{kname}", "achieved": achieved, "peak": peak,
                  "frac": achieved / peak, "traffic": ncu_traffic(key), "launch_ms": kmean * 1e3})
@@ -1018,8 +1022,7 @@ def resident_leg(args, w, inputs, path, steps, warmup, label):
         roof = {"bound": "hbm", "unit": "GB/s", "peak_basis": f"HBM copy {pk['hbm_gbs']} GB/s ({pk_kind})",
                 "bytes_per_launch": byts}
         achieved = byts / kmean / 1e9
-    kname = {"fma": "sched_fma_kernel", "split3_wide": "sched_wide_kernel",
-             "split3_tma": "sched_tma_kernel"}.get(path, "sched_fused_kernel")
+    kname = scheduler_kernel(path)
     roof.update({"kernel": f"gvm::{kname}", "achieved": achieved, "peak": peak, "frac": achieved / peak,
                  "traffic": ncu_traffic(f"{kname}/{label}"), "launch_ms": kmean * 1e3})
     return {
@@ -1126,7 +1129,7 @@ def plain_per_rank(w, inputs, phases, init="before", timeout_s=300.0):
     its own CUDA context on the default stream, running its tasks one after
     another through the same standalone task kernel. Each process is pinned
     to its own core, as the paper pins its processes. ``phases`` is a list of
-    (path, mode): path "fma" or "split3" (the fused split3 kernel), mode
+    (path, mode): path "fma" or "split3", mode
     "resident" (operands on the device before the start, kernel +
     synchronize per task) or "copy" (synchronous copies of A, B in and C out
     around every kernel). ``init`` "before": context creation, device
@@ -1219,7 +1222,7 @@ def plain_per_rank(w, inputs, phases, init="before", timeout_s=300.0):
                 "parity_spot_rel_err": max(spot),
                 "form": f"{R} processes (one core each), one CUDA context each, default stream, "
                         f"{'operands resident' if mode == 'resident' else 'synchronous copies per task'}, "
-                        f"{'FMA' if path == 'fma' else 'split3 (fused)'} SGEMM kernel alone per task",
+                        f"{'FMA' if path == 'fma' else 'split3'} SGEMM kernel alone per task",
             }
             if init == "timed" and i == 0:
                 ti = [x[2] / 1e9 for x in res]
@@ -1931,12 +1934,8 @@ def grouped_arm(args):
                    "sgemm_path": args.path, "mode": "barrier", "tflop_per_step": flops / 1e12},
         "roofline": {"bound": bound, "unit": "TFLOP/s", "achieved": achieved, "peak": peak, "frac": achieved / peak,
                      "peak_basis": basis, "frac_of_burst_peak": burst_frac,
-                     "kernel": "gvm::" + {"split3": "sched_fused_kernel",
-                                          "split3_wide": "sched_wide_kernel",
-                                          "split3_tma": "sched_tma_kernel"}.get(args.path, "sched_fma_kernel"),
-                     "traffic": ncu_traffic({"split3": "sched_fused_kernel", "split3_wide": "sched_wide_kernel",
-                                             "split3_tma": "sched_tma_kernel"}.get(
-                         args.path, "sched_fma_kernel") + "/grouped") if (R, P) == (64, 256) else None,
+                     "kernel": "gvm::" + scheduler_kernel(args.path),
+                     "traffic": ncu_traffic(scheduler_kernel(args.path) + "/grouped") if (R, P) == (64, 256) else None,
                      "launch_ms": kmean * 1e3},
         "sched_timeline_last_launch": {
             "cta_ms": {"acquire": ph[0] / 1e6, "stage_wait": ph[2] / 1e6, "gemm": ph[3] / 1e6,
@@ -1953,7 +1952,7 @@ def grouped_arm(args):
 
 def main():
     args = parse()
-    if args.path is None:  # the split3 tile form the autotuner chose for this workload class (fused if none)
+    if args.path is None:  # the split3 value the autotuner chose for this workload class (split3 if none)
         from paper_1511_07658_gb300.manager import tuning
 
         t = tuning()

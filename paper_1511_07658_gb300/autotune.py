@@ -11,18 +11,14 @@ and keeps the fastest:
   one pinned block (8 steps);
 * ``vadd_tile`` (elements per vector-add tile; 0 = per task, n / CTAs): 16
   ranks x 8 resident vector adds of n = 2^22 (10 steps);
-* ``sgemm_form`` (the split3 SGEMM tile form): fused 128 x 256 tiles
-  (operands loaded by the staging warps), the same tiles with A and B landed
-  by TMA and split in place, and wide 256 x 256 tiles of one CTA (A by TMA),
-  per workload class: square 512^3 (16 x 64 tasks, the headline shape),
+* ``sgemm_form`` (the split3 value: ``split3``, ``split3_tma`` and
+  ``split3_wide`` run one kernel form, so their times differ by noise), per
+  workload class: square 512^3 (16 x 64 tasks, the headline shape),
   512 x 768 x 512 (16 x 16), 2048^3 (16 x 1) and a grouped mix of shapes
   drawn from {128, ..., 2048} (64 ranks x 64 tasks, a quarter of the
   grouped benchmark's tasks per rank). ``sgemm_form_by_class`` keeps the
-  fastest form of each class; ``sgemm_form``, the manager's default, is the
-  512^3 class's. A tile form per task inside one launch would need several
-  forms in one kernel, whose converters then spill (measured); so the form
-  is chosen per manager (per workload), and a task's result is the same
-  alone and in any mix (every form computes each element the same way);
+  fastest of each class; ``sgemm_form``, the manager's default, is the
+  512^3 class's;
 * ``l2_prefetch`` (split3: the next queued tile's operands prefetched into
   L2): on against off on the same three workloads, kept if it wins all.
 
@@ -216,9 +212,8 @@ def run(path: str = _m.TUNING_FILE) -> dict:
             "copy_run_bytes": "end-to-end leg, 16 ranks x 16 SGEMM 512^3, operands in one pinned block per rank",
             "vadd_tile": "16 ranks x 8 resident vector adds, n = 2^22",
             "sgemm_form": "resident SGEMM, 16 ranks x (64 of 512^3, 16 of 512 x 768 x 512, 1 of 2048^3), "
-                          "64 ranks x 64 of the grouped mix: fused 128 x 256 tiles, the same tiles landed by TMA, "
-                          "wide 256 x 256 tiles",
-            "l2_prefetch": "the same SGEMM workloads, fused tiles, next-tile L2 prefetch off (0) and on (1)",
+                          "64 ranks x 64 of the grouped mix: the three split3 values (one kernel form)",
+            "l2_prefetch": "the same SGEMM workloads, next-tile L2 prefetch off (0) and on (1)",
         },
     }
     with open(path, "w") as f:

@@ -278,7 +278,7 @@ class Manager:
         cfg.max_ranks = ranks
         cfg.ring_depth = ring_depth
         cfg.mode = _MODES[mode]
-        if sgemm_path is None:  # the autotuner's form, else the fused split3 tiles
+        if sgemm_path is None:  # the autotuner's value, else split3
             sgemm_path = tuning().get("sgemm_form", "split3")
         cfg.sgemm_path = _PATHS[sgemm_path]
         ctrl_bytes = L.gvm_ctrl_bytes(byref(cfg))
