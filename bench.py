@@ -72,7 +72,7 @@ def parse():
     p.add_argument("--duration", type=float, default=10.0,
                    help="stress: seconds of arrivals per load point (the configuration's is 60)")
     p.add_argument("--path", choices=["split3", "split3_wide", "split3_tma", "fma"], default=None,
-                   help="SGEMM arithmetic and tile form (default: the autotuner's split3 form)")
+                   help="SGEMM arithmetic (the split3 values run one kernel form; default: the autotuner's)")
     p.add_argument("--mode", choices=["barrier", "continuous"], default="barrier")
     p.add_argument("--skip-e2e", action="store_true")
     p.add_argument("--skip-cpu", action="store_true")
