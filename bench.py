@@ -219,7 +219,7 @@ def peaks():
 
 # The sources the scheduler kernels are compiled from (host code does not
 # change their DRAM traffic per tile).
-KERNEL_SOURCES = ("gvm_sched.cu", "gvm_pair.cuh", "gvm_device.cuh", "gvm_internal.h")
+KERNEL_SOURCES = ("gvm_sched.cu", "gvm_pair.cuh", "gvm_ring.h", "gvm_device.cuh", "gvm_internal.h")
 
 
 def scheduler_kernel(path):

@@ -40,7 +40,8 @@ __global__ void __launch_bounds__(kFmaThreads, 2) fma_sgemm_kernel(const float* 
 
 // Pair form: a persistent grid of clusters of two CTAs; cluster i takes tiles
 // i, i + clusters, ... (row-major over the tile grid). Every role walks the
-// same sequence.
+// same sequence. k-steps are numbered through: 65536^3 has 1.8 million for
+// each of 76 clusters, far from the wrap of a 32-bit number.
 struct PrStandShared {
   PrShared ps;
   uint32_t abort_flag, fail_where;

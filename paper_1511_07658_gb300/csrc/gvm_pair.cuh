@@ -61,6 +61,7 @@
 #pragma once
 
 #include "gvm_device.cuh"
+#include "gvm_ring.h"
 
 namespace gvm {
 
@@ -72,9 +73,7 @@ constexpr int kPrN = 256;  // most columns of a pair tile (half per CTA)
 // stage's own it would wait for the same parity each time, and a parity does
 // not tell a phase from the one two before it.)
 constexpr int kPrLand = 4;
-constexpr int kPrStages = 3;
-constexpr int kPrBars = 6;
-static_assert(kPrLand % 2 == 0 && kPrBars == 2 * kPrStages, "a group sees every phase of its barriers");
+static_assert(kPrLand % 2 == 0 && kPrBars % 2 == 0, "a group sees every phase of its barriers");
 // Packed operands take more room in a landing, so that tiles with one have
 // at most kPrPackedN columns.
 constexpr int kPrPackedN = 192;
@@ -326,8 +325,8 @@ __device__ __forceinline__ void pr_init(PrShared* ps) {
       mbar_init(&ps->landed[i], 1);
       mbar_init(&ps->land_free[i], kPrGroupWarps);
     }
-    for (int i = 0; i < kPrBars; ++i) mbar_init(&ps->empty[i], 1);
-    for (int s = 0; s < kPrStages; ++s) mbar_init(&ps->full[s], 2 * kPrGroupWarps);
+    for (uint32_t i = 0; i < kPrBars; ++i) mbar_init(&ps->empty[i], 1);
+    for (uint32_t s = 0; s < kPrStages; ++s) mbar_init(&ps->full[s], 2 * kPrGroupWarps);
     for (int b = 0; b < 2; ++b) {
       mbar_init(&ps->acc_full[b], 1);
       mbar_init(&ps->acc_empty[b], 2 * kPrEpiWarps);
@@ -461,8 +460,8 @@ __device__ __forceinline__ bool pr_wait_landed(PrShared* ps, uint32_t ql, uint64
 // Converter warps, k-step q: the MMAs have read its stage's previous k-step, q - 3.
 __device__ __forceinline__ bool pr_wait_stage(PrShared* ps, uint32_t q, uint64_t timeout_ns, uint32_t* cta_abort,
                                               uint32_t* fail_where) {
-  if (q < kPrStages || mbar_wait_warp<false>(&ps->empty[(q - kPrStages) % kPrBars], ((q - kPrStages) / kPrBars) & 1u,
-                                             timeout_ns, cta_abort))
+  if (!pr_stage_used(q) || mbar_wait_warp<false>(&ps->empty[pr_empty_bar(q - kPrStages)], pr_empty_parity(q - kPrStages),
+                                                 timeout_ns, cta_abort))
     return true;
   if ((threadIdx.x & 31) == 0) pr_fail(ps, cta_abort, fail_where, kWhereFullBarrier);
   return false;
@@ -489,7 +488,7 @@ __device__ __forceinline__ bool pr_convert_aligned(const PrTile t, uint32_t land
   const uint32_t wr = swz64(r, c);
   for (int kb = (int)((it + (uint32_t)par) & 1u); kb < nkb; kb += 2) {
     const uint32_t q = it + (uint32_t)kb, ql = it_l + (uint32_t)kb;
-    const uint32_t s = q % kPrStages, i = ql % kPrLand;
+    const uint32_t s = pr_stage(q), i = ql % kPrLand;
     if (!pr_wait_landed(ps, ql, timeout_ns, cta_abort, fail_where)) return false;
     const uint32_t ld = land0 + i * kPrLandBytes;
     const uint32_t st = st0 + s * kPrStageBytes;
@@ -584,7 +583,7 @@ __device__ __forceinline__ bool pr_convert_packed(const PrTile t, uint32_t land0
   const uint32_t wr = swz64(r, c);
   for (int kb = (int)((it + (uint32_t)par) & 1u); kb < nkb; kb += 2) {
     const uint32_t q = it + (uint32_t)kb, ql = it_l + (uint32_t)kb;
-    const uint32_t s = q % kPrStages, i = ql % kPrLand;
+    const uint32_t s = pr_stage(q), i = ql % kPrLand;
     if (!pr_wait_landed(ps, ql, timeout_ns, cta_abort, fail_where) ||
         !pr_wait_stage(ps, q, timeout_ns, cta_abort, fail_where))
       return false;
@@ -798,7 +797,7 @@ __device__ __forceinline__ bool pr_mma(const PrTile t, uint8_t* stages, PrShared
   const int nkb = (t.k + kTcBK - 1) / kTcBK;
   const uint32_t st0 = smem_u32(stages);
   for (int kb = 0; kb < nkb; ++kb) {
-    const uint32_t q = it + (uint32_t)kb, s = q % kPrStages, ph = (q / kPrStages) & 1u;
+    const uint32_t q = it + (uint32_t)kb, s = pr_stage(q), ph = pr_full_parity(q);
     const long long c0 = wait_acc != nullptr ? clock64() : 0;
     if (!mbar_wait(&ps->full[s], ph, timeout_ns, cta_abort)) {
       pr_fail(ps, cta_abort, fail_where, kWhereFullBarrier);
@@ -817,7 +816,7 @@ __device__ __forceinline__ bool pr_mma(const PrTile t, uint8_t* stages, PrShared
       umma_bf16_pair(tmem, dAh + adv_a, dBl + adv_b, idesc, 1u);
       umma_bf16_pair(tmem, dAh + adv_a, dBh + adv_b, idesc, 1u);
     }
-    umma_commit_pair(&ps->empty[q % kPrBars]);
+    umma_commit_pair(&ps->empty[pr_empty_bar(q)]);
   }
   umma_commit_pair(&ps->acc_full[b]);
   return true;

@@ -871,7 +871,7 @@ PAIR_ROLE pair_mma(const SchedParams& p, PairSchedShared& sh, uint8_t* stages) {
       report_error(p, kStatusTimeout, sh.fail_where, seq);
       break;
     }
-    it_k += (uint32_t)((t.k + kTcBK - 1) / kTcBK);
+    it_k = pr_next_first(it_k, (uint32_t)((t.k + kTcBK - 1) / kTcBK));
     ++tile_no;
   }
 }
@@ -942,7 +942,7 @@ PAIR_ROLE pair_convert(const SchedParams& p, PairSchedShared& sh, uint8_t* land,
       if (lane == 0) pair_item_release(sh, seq);
       ok = pr_convert(t, land, stages, &sh.ps, it_k, it_l, p.wait_timeout_ns, &sh.abort, &sh.fail_where);
       const uint32_t nkb = (uint32_t)((t.k + kTcBK - 1) / kTcBK);
-      it_k += nkb;
+      it_k = pr_next_first(it_k, nkb);
       it_l += nkb;
       if (prof) sh.prof[kProfGemm] += globaltimer() - t0;
     } else if (kind == kTaskVadd || kind == kTaskVmul) {
