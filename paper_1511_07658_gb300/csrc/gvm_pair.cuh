@@ -24,7 +24,7 @@
 //                into C, while the next tile's MMAs fill the other one;
 //   warps 4-11   converters, two groups of four warps taking alternate k-steps;
 //   warp 12      MMA issue (one thread, in the even CTA -- the leader -- only);
-//   warp 13      the scheduler's tile claims (leader; idle otherwise);
+//   warp 13      the scheduler's tile claims (leader) and their slots' return (peer);
 //   warp 14      producer: one thread issues the tensor copies.
 // The single threads are elected with elect.sync: the compiler then keeps
 // their operands in uniform registers. Picked by lane == 0, an MMA took 133

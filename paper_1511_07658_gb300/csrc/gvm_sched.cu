@@ -672,7 +672,8 @@ __global__ void __launch_bounds__(kFmaThreads, 2) sched_fma_kernel(const __grid_
 // CTAs stage their halves of the operands, the leader issues the MMAs, each
 // CTA's epilogue warps store its 128 rows. A vector tile is split in two
 // halves, each run by a CTA's converter and epilogue warps. Either way each
-// CTA counts its half, so a task is complete after 2 x ntiles counts. No warp
+// CTA counts its half, so a task is complete after 2 x ntiles counts. The
+// peer's control warp hands read items back to the leader. No warp
 // waits for another warp's tile except through the pipeline's barriers.
 
 constexpr int kItems = 4;                               // items in flight between the control warp and the others
@@ -724,7 +725,7 @@ __device__ __forceinline__ void prefetch_task_operands(const Item& it, int64_t t
 struct PairSchedShared {
   PrShared ps;
   uint64_t item_full[kItems];   // each CTA: control -> its consumers
-  uint64_t item_empty[kItems];  // leader: consumers of both CTAs -> control
+  uint64_t item_empty[kItems];  // leader: its consumers and the peer's relay -> control; peer: its consumers -> relay
   PrItem items[kItems];
   uint32_t fin[kFinSlots];        // warps of this CTA done with item (seq % kFinSlots)
   uint32_t abort;
@@ -783,8 +784,9 @@ __device__ __forceinline__ bool pair_item_wait(const SchedParams& p, PairSchedSh
   }
   return false;
 }
+// To the CTA's own barrier: see pair_relay.
 __device__ __forceinline__ void pair_item_release(PairSchedShared& sh, uint32_t seq) {
-  mbar_arrive_cta(&sh.item_empty[seq % kItems], 0);
+  mbar_arrive(&sh.item_empty[seq % kItems]);
 }
 
 // The roles, each a function of its own: ptxas gives a function the registers
@@ -836,6 +838,33 @@ PAIR_ROLE pair_control(const SchedParams& p, PairSchedShared& sh) {
     }
     __syncwarp();
     if (got == 0) break;
+  }
+}
+
+// Relay (peer's control warp, one thread): hands the slots that this CTA's
+// consumers have read back to the leader. The leader overwrites them from
+// another CTA, which a CTA-scope release does not order after the reads, and a
+// cluster-scope one by each consumer waits for its other accesses under way:
+// 64 vector adds of 2^22 took 6% longer so, the grouped mix 2%. Here the
+// consumers release to their own CTA, and this thread, with no accesses of its
+// own, passes what it has acquired from them on to the cluster.
+PAIR_ROLE pair_relay(const SchedParams& p, PairSchedShared& sh) {
+  for (uint32_t seq = 0; pair_item_wait<false>(p, sh, seq); ++seq) {
+    const uint32_t slot = seq % kItems, kind = sh.items[slot].kind;
+    // The control warp waits for a slot only once it wants it again, this thread
+    // from the item's posting on, up to kItems items earlier.
+    bool ok = false;
+    for (int i = 0; i <= kItems && !ok && !sh.abort; ++i)
+      ok = mbar_wait(&sh.item_empty[slot], (seq / kItems) & 1u, p.wait_timeout_ns, &sh.abort);
+    if (!ok) {
+      if (!sh.abort) {
+        pr_fail(&sh.ps, &sh.abort, &sh.fail_where, kWhereItemRing);
+        report_error(p, kStatusTimeout, kWhereItemRing, seq);
+      }
+      break;
+    }
+    mbar_arrive_release_cta(&sh.item_empty[slot], 0);
+    if (kind == kItemExit) break;
   }
 }
 
@@ -1024,8 +1053,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPrThreads, 1)
     for (int i = 0; i < kFinSlots; ++i) sh.fin[i] = 0;
     for (int i = 0; i < kItems; ++i) {
       mbar_init(&sh.item_full[i], kItemFields + 1);  // a lane per 16-byte piece
-      // Each CTA's epilogue and converter warps and producer; the leader's MMA thread.
-      mbar_init(&sh.item_empty[i], 2 * (kPrEpiWarps + kPrConvWarps + 1) + 1);
+      // The CTA's epilogue and converter warps and producer; leader: the MMA thread and the peer's relay.
+      mbar_init(&sh.item_empty[i], kPrEpiWarps + kPrConvWarps + 1 + (cluster_ctarank() == 0 ? 2 : 0));
     }
     Claim* cl = reinterpret_cast<Claim*>(sh.claim);
     cl->has_resv = 0;
@@ -1054,6 +1083,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPrThreads, 1)
     if (tid == 32 * kPrCtlWarp) reinterpret_cast<Claim*>(sh.claim)->hint = first;
     __syncwarp();
     pair_control(p, sh);
+  } else if (elect_one()) {
+    pair_relay(p, sh);
   }
   __syncwarp();
   pr_teardown(&sh.ps, 2 * p.wait_timeout_ns);
