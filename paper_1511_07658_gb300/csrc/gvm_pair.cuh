@@ -561,9 +561,9 @@ __device__ __forceinline__ bool pr_convert_packed(const PrTile t, uint32_t land0
   const int par = cw / kPrGroupWarps, w = cw % kPrGroupWarps;
   const int nkb = (t.k + kTcBK - 1) / kTcBK;
   const int slabs = t.ncols >> 6, m = t.m, k = t.k;
-  const int64_t n = t.n;
+  const int n = (int)t.n;
   const int row0 = t.row0 + (int)ps->cta * 128;
-  const int64_t col0 = t.col0 + (int64_t)((int)ps->cta * (t.ncols >> 1));
+  const int col0 = (int)t.col0 + (int)ps->cta * (t.ncols >> 1);
   const bool has_a = row0 < m;
   const bool map_a = (t.land & kPrMapA) != 0, map_b = (t.land & kPrMapB) != 0;
   const bool pack_a = !map_a || (t.land & kPrPackedA) != 0, pack_b = !map_b || (t.land & kPrPackedB) != 0;
@@ -601,7 +601,7 @@ __device__ __forceinline__ bool pr_convert_packed(const PrTile t, uint32_t land0
       }
     };
     // 8 values of a row from global memory, zero outside the matrix.
-    auto fetch = [](const float* src, bool row_in, int64_t left, float (&v)[8]) {
+    auto fetch = [](const float* src, bool row_in, int left, float (&v)[8]) {
 #pragma unroll
       for (int e = 0; e < 8; ++e) v[e] = (row_in && e < left) ? __ldcg(src + e) : 0.f;
     };
@@ -649,7 +649,7 @@ __device__ __forceinline__ bool pr_convert_packed(const PrTile t, uint32_t land0
         const int b = b0 + u;
         if (b < slabs) {
           if (pack_b && kr >= full_k) {
-            const int64_t col = col0 + 32 * b + 8 * (int)c;
+            const int col = col0 + 32 * b + 8 * (int)c;
             fetch(B + (int64_t)kr * n + col, kr < k, n - col, x[u]);
           }
           const uint32_t at = st + (uint32_t)w * kPrBAtomK + (uint32_t)b * kPrBAtomN + wr;
@@ -734,9 +734,12 @@ __device__ __forceinline__ bool pr_vec_produce(const float* a, const float* b, i
   return true;
 }
 
-// Converter warps: c = a op b over the landings of this warp's group.
+// Converter warps: c = a op b over the landings of this warp's group. Whole
+// landings run unrolled. A function of its own: inlined into the converters'
+// role, its code changed with the product loops beside it (64 vector adds of
+// 2^22 493 to 507 us a launch, multiplies 593 to 630; now 496 and 555).
 template <int OP>
-__device__ __forceinline__ bool pr_vec_convert(const float* a, const float* b, float* c, int64_t len, int iters,
+static __device__ __noinline__ bool pr_vec_convert(const float* a, const float* b, float* c, int64_t len, int iters,
                                                uint8_t* land, PrShared* ps, uint32_t it_l, uint64_t timeout_ns,
                                                uint32_t* cta_abort, uint32_t* fail_where) {
   const int cw = (int)(threadIdx.x >> 5) - kPrConvWarp0, lane = threadIdx.x & 31;
@@ -752,19 +755,29 @@ __device__ __forceinline__ bool pr_vec_convert(const float* a, const float* b, f
     const int64_t at = (int64_t)ch * kPrVecChunk, left = len - at;
     const uint32_t n4 = left >= kPrVecChunk ? kPrVecChunk / 4 : left > 0 ? (uint32_t)(left >> 2) : 0u;
     const uint32_t st = land0 + (q % kPrLand) * kPrLandBytes + 16u * t;
-#pragma unroll 4
-    for (uint32_t i = t, o = 0; i < n4; i += 32 * kPrGroupWarps, o += 16u * 32 * kPrGroupWarps) {
-      const uint4 xu = ld_shared_v4(st + o), yu = ld_shared_v4(st + kPrVecB + o);
-      const float4 x = *reinterpret_cast<const float4*>(&xu), y = *reinterpret_cast<const float4*>(&yu);
-      const float4 z = elem_op4<OP>(x, y, iters);
-      float* dst = c + at + 4 * (int64_t)i;
-      if (cvec) {
-        __stcs(reinterpret_cast<float4*>(dst), z);
-      } else {
-        dst[0] = z.x;
-        dst[1] = z.y;
-        dst[2] = z.z;
-        dst[3] = z.w;
+    auto four = [&](uint32_t j) {  // the thread's j-th four elements
+      const uint4 xu = ld_shared_v4(st + j * (16u * 32 * kPrGroupWarps));
+      const uint4 yu = ld_shared_v4(st + kPrVecB + j * (16u * 32 * kPrGroupWarps));
+      return elem_op4<OP>(*reinterpret_cast<const float4*>(&xu), *reinterpret_cast<const float4*>(&yu), iters);
+    };
+    float* dst = c + at + 4 * (int64_t)t;
+    constexpr uint32_t kAll = kPrVecChunk / (4 * 32 * kPrGroupWarps);
+    if (cvec && left >= kPrVecChunk) {
+#pragma unroll 8
+      for (uint32_t j = 0; j < kAll; ++j) __stcs(reinterpret_cast<float4*>(dst + j * (4 * 32 * kPrGroupWarps)), four(j));
+    } else {
+#pragma unroll 1
+      for (uint32_t j = 0; t + j * (32 * kPrGroupWarps) < n4; ++j) {
+        const float4 z = four(j);
+        float* d = dst + j * (4 * 32 * kPrGroupWarps);
+        if (cvec) {
+          __stcs(reinterpret_cast<float4*>(d), z);
+        } else {
+          d[0] = z.x;
+          d[1] = z.y;
+          d[2] = z.z;
+          d[3] = z.w;
+        }
       }
     }
     if (left > 0 && left < kPrVecChunk) {  // the last elements, not landed

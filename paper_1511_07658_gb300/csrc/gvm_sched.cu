@@ -686,7 +686,7 @@ struct alignas(16) PrItem {
   uint32_t kind;  // kItemExit, kItemNop or a task type
   uint32_t task;
   uint32_t tile;
-  uint32_t pad;
+  uint32_t first;  // SGEMM: number of the tile's first k-step (gvm_ring.h)
   uint32_t type, flags, rank, slot;
   uint32_t tag, ntiles, nsplit, tiles_m;
   uint32_t tiles_n, kp;
@@ -697,6 +697,8 @@ struct alignas(16) PrItem {
   uint64_t a, b, c, scratch;
 };
 constexpr int kItemFields = 6;  // 16-byte pieces of task fields
+constexpr int kItemFieldK = 2;  // the one that ends with k
+static_assert(offsetof(TaskBody, k) == kFieldsAt + 16 * kItemFieldK + 12, "k's place");
 static_assert(sizeof(PrItem) == 16 * (kItemFields + 1) && offsetof(TaskBody, c) - offsetof(TaskBody, type) ==
                   offsetof(PrItem, c) - offsetof(PrItem, type), "item = header + task fields");
 
@@ -800,6 +802,9 @@ PAIR_ROLE pair_control(const SchedParams& p, PairSchedShared& sh) {
   const int lane = threadIdx.x & 31;
   Claim* cl = reinterpret_cast<Claim*>(sh.claim);
   const uint64_t to = p.wait_timeout_ns;
+  // k-step numbers are counted here and posted with the items: one register
+  // less in the converters, whose loops spill.
+  uint32_t first = 0;
   for (uint32_t seq = 0;; ++seq) {
     const uint32_t slot = seq % kItems, ph = (seq / kItems) & 1u;
     uint32_t ok = 1;
@@ -818,17 +823,19 @@ PAIR_ROLE pair_control(const SchedParams& p, PairSchedShared& sh) {
     const int got = sh.abort ? 0 : acquire<true>(p, cl, sh.list, task, tile, sh.prof, true, to / 4);
     // Lanes 0..5 carry the task's fields, lane 6 the header (it reads the piece
     // that begins with the type), to both CTAs.
+    uint4 v = make_uint4(got == 2 ? kItemNop : kItemExit, 0, 0, 0);
+    if (got == 1 && lane <= kItemFields)
+      v = ld_cg_v4(reinterpret_cast<const uint8_t*>(&p.tasks[task].body) + kFieldsAt + 16 * (lane % kItemFields));
+    const uint32_t kind = __shfl_sync(0xffffffffu, v.x, 0), k = __shfl_sync(0xffffffffu, v.w, kItemFieldK);
     if (lane <= kItemFields) {
-      uint4 v = make_uint4(got == 2 ? kItemNop : kItemExit, 0, 0, 0);
-      if (got == 1)
-        v = ld_cg_v4(reinterpret_cast<const uint8_t*>(&p.tasks[task].body) + kFieldsAt + 16 * (lane % kItemFields));
-      if (lane == kItemFields && got == 1) v = make_uint4(v.x, task, tile, 0);
+      if (lane == kItemFields && got == 1) v = make_uint4(v.x, task, tile, first);
       uint4* dst = reinterpret_cast<uint4*>(&sh.items[slot]) + (lane == kItemFields ? 0 : lane + 1);
       *dst = v;
       st_cluster_v4(mapa_shared(smem_u32(dst), 1), v);
       mbar_arrive_release_cta(&sh.item_full[slot], 1);
       mbar_arrive(&sh.item_full[slot]);
     }
+    if (got == 1 && kind == kTaskSgemm) first = pr_next_first(first, (k + kTcBK - 1) / kTcBK);
     __syncwarp();
     if (lane == 0) {
       sh.prof[kProfAcquire] += globaltimer() - t0;
@@ -887,20 +894,19 @@ __device__ __forceinline__ bool pair_vec_lands(const PrItem& it) { return ((it.a
 
 // MMA issue (leader, one thread): GEMM items only; every item is read and released.
 PAIR_ROLE pair_mma(const SchedParams& p, PairSchedShared& sh, uint8_t* stages) {
-  uint32_t it_k = 0, tile_no = 0;
+  uint32_t tile_no = 0;
   for (uint32_t seq = 0; pair_item_wait<false>(p, sh, seq); ++seq) {
     const PrItem& item = sh.items[seq % kItems];
-    const uint32_t kind = item.kind;
+    const uint32_t kind = item.kind, first = item.first;
     const PrTile t = kind == kTaskSgemm ? pair_tile(item) : PrTile{};
     pair_item_release(sh, seq);
     if (kind == kItemExit) break;
     if (kind != kTaskSgemm) continue;
-    if (!pr_mma(t, stages, &sh.ps, it_k, tile_no, p.wait_timeout_ns, &sh.abort, &sh.fail_where,
+    if (!pr_mma(t, stages, &sh.ps, first, tile_no, p.wait_timeout_ns, &sh.abort, &sh.fail_where,
                 &sh.prof[kProfMmaWait])) {
       report_error(p, kStatusTimeout, sh.fail_where, seq);
       break;
     }
-    it_k = pr_next_first(it_k, (uint32_t)((t.k + kTcBK - 1) / kTcBK));
     ++tile_no;
   }
 }
@@ -959,7 +965,7 @@ __device__ __forceinline__ void pair_vector(const SchedParams& p, PairSchedShare
 PAIR_ROLE pair_convert(const SchedParams& p, PairSchedShared& sh, uint8_t* land, uint8_t* stages) {
   const int lane = threadIdx.x & 31;
   const bool prof = threadIdx.x == kPrConvWarp0 * 32;
-  uint32_t it_k = 0, it_l = 0;
+  uint32_t it_l = 0;
   for (uint32_t seq = 0; pair_item_wait<true>(p, sh, seq); ++seq) {
     const PrItem& item = sh.items[seq % kItems];
     const uint32_t kind = item.kind;
@@ -967,12 +973,11 @@ PAIR_ROLE pair_convert(const SchedParams& p, PairSchedShared& sh, uint8_t* land,
     bool ok = true;
     if (kind == kTaskSgemm) {
       const PrTile t = pair_tile(item);
+      const uint32_t first = item.first;
       __syncwarp();
       if (lane == 0) pair_item_release(sh, seq);
-      ok = pr_convert(t, land, stages, &sh.ps, it_k, it_l, p.wait_timeout_ns, &sh.abort, &sh.fail_where);
-      const uint32_t nkb = (uint32_t)((t.k + kTcBK - 1) / kTcBK);
-      it_k = pr_next_first(it_k, nkb);
-      it_l += nkb;
+      ok = pr_convert(t, land, stages, &sh.ps, first, it_l, p.wait_timeout_ns, &sh.abort, &sh.fail_where);
+      it_l += (uint32_t)((t.k + kTcBK - 1) / kTcBK);
       if (prof) sh.prof[kProfGemm] += globaltimer() - t0;
     } else if (kind == kTaskVadd || kind == kTaskVmul) {
       if (pair_vec_lands(item)) {
