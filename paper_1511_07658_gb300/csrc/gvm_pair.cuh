@@ -536,6 +536,7 @@ __device__ __forceinline__ bool pr_convert_aligned(const PrTile t, uint32_t land
     // value equals both constants, which the compiler does not see).
     const uint32_t last = xb[0][1].w ^ xb[1][1].w ^ xb[2][1].w ^ xb[3][1].w;
     const bool read = (__ballot_sync(0xffffffffu, last == 0x7fa5a5a5u) & __ballot_sync(0xffffffffu, last == 0x7f5a5a5au)) == 0;
+    __syncwarp();  // orders the other lanes' reads before lane 0's arrive
     if (lane == 0 && read) mbar_arrive(&ps->land_free[i]);
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
