@@ -807,10 +807,16 @@ PAIR_ROLE pair_control(const SchedParams& p, PairSchedShared& sh) {
   uint32_t first = 0;
   for (uint32_t seq = 0;; ++seq) {
     const uint32_t slot = seq % kItems, ph = (seq / kItems) & 1u;
-    uint32_t ok = 1;
-    if (lane == 0) ok = mbar_wait_cluster(&sh.item_empty[slot], ph ^ 1u, to, &sh.abort) ? 1u : 0u;
-    if (!__shfl_sync(0xffffffffu, ok, 0)) {
-      if (lane == 0 && !sh.abort) {
+    // One lane waits and reads the abort word, and all go by what it found: the
+    // claim below is warp-collective, and another warp may set the word meanwhile.
+    uint32_t seen = 0;  // bit 0: the slot is free, bit 1: the CTA stops
+    if (lane == 0) {
+      seen = mbar_wait_cluster(&sh.item_empty[slot], ph ^ 1u, to, &sh.abort) ? 1u : 0u;
+      if (ld_volatile_u32(&sh.abort)) seen |= 2u;
+    }
+    seen = bcast(seen);
+    if (!(seen & 1u)) {
+      if (lane == 0 && !(seen & 2u)) {
         pr_fail(&sh.ps, &sh.abort, &sh.fail_where, kWhereItemRing);
         report_error(p, kStatusTimeout, kWhereItemRing, seq);
       }
@@ -820,7 +826,7 @@ PAIR_ROLE pair_control(const SchedParams& p, PairSchedShared& sh) {
     uint32_t task = 0, tile = 0;
     // An idle control warp posts a no-op item now and then, so that the
     // other warps' waits for items stay bounded.
-    const int got = sh.abort ? 0 : acquire<true>(p, cl, sh.list, task, tile, sh.prof, true, to / 4);
+    const int got = (seen & 2u) ? 0 : acquire<true>(p, cl, sh.list, task, tile, sh.prof, true, to / 4);
     // Lanes 0..5 carry the task's fields, lane 6 the header (it reads the piece
     // that begins with the type), to both CTAs.
     uint4 v = make_uint4(got == 2 ? kItemNop : kItemExit, 0, 0, 0);

@@ -25,6 +25,8 @@ def body(name, function):
         # released to the peer's own barrier, and from there to the cluster.
         ("gvm_sched.cu", "pair_item_release", r"mbar_arrive\(&sh\.item_empty"),
         ("gvm_sched.cu", "pair_relay", r"mbar_wait\(&sh\.item_empty.*mbar_arrive_release_cta\(&sh\.item_empty"),
+        # One lane's reading of the abort word decides for the warp that claims together.
+        ("gvm_sched.cu", "pair_control", r"seen = bcast\(seen\);(?!.*sh\.abort \?).*\(seen & 2u\) \? 0 : acquire<true>"),
         # Every lane's reads of a landing before lane 0 frees it for the next copies.
         ("gvm_pair.cuh", "pr_convert_aligned", r"read_b\(3\);.*__syncwarp\(\);\s*if \([^)]*\) mbar_arrive\(&ps->land_free"),
         ("gvm_pair.cuh", "pr_convert_packed", r"__syncwarp\(\);\s*if \([^)]*\) \{\s*mbar_arrive\(&ps->land_free"),
