@@ -249,8 +249,7 @@ __device__ __forceinline__ float ld_stream(const float* p) {
   return kL2 ? __ldcg(p) : *p;
 }
 
-// U: float4 loads of each operand in flight a thread.
-template <int OP, bool kL2, int U>
+template <int OP, bool kL2>
 __device__ __forceinline__ void elementwise_range(const float* __restrict__ a, const float* __restrict__ b,
                                                   float* __restrict__ c, int64_t lo, int64_t hi, int tid, int nthr,
                                                   int iters) {
@@ -259,6 +258,7 @@ __device__ __forceinline__ void elementwise_range(const float* __restrict__ a, c
                     15) == 0;
   int64_t done = lo;
   if (vec) {
+    constexpr int U = 4;  // loads of each operand in flight a thread
     const int64_t nv = (hi - lo) >> 2;
     const float4* a4 = reinterpret_cast<const float4*>(a + lo);
     const float4* b4 = reinterpret_cast<const float4*>(b + lo);
@@ -281,16 +281,16 @@ __device__ __forceinline__ void elementwise_range(const float* __restrict__ a, c
   for (int64_t i = done + tid; i < hi; i += nthr) c[i] = elem_op<OP>(ld_stream<kL2>(a + i), ld_stream<kL2>(b + i), iters);
 }
 
-template <bool kL2 = false, int U = 4>
+template <bool kL2 = false>
 __device__ __forceinline__ void vadd_range(const float* __restrict__ a, const float* __restrict__ b,
                                            float* __restrict__ c, int64_t lo, int64_t hi, int tid, int nthr) {
-  elementwise_range<kElemAdd, kL2, U>(a, b, c, lo, hi, tid, nthr, 0);
+  elementwise_range<kElemAdd, kL2>(a, b, c, lo, hi, tid, nthr, 0);
 }
-template <bool kL2 = false, int U = 4>
+template <bool kL2 = false>
 __device__ __forceinline__ void vmul_range(const float* __restrict__ a, const float* __restrict__ b,
                                            float* __restrict__ c, int64_t lo, int64_t hi, int tid, int nthr,
                                            int iters) {
-  elementwise_range<kElemMul, kL2, U>(a, b, c, lo, hi, tid, nthr, iters);
+  elementwise_range<kElemMul, kL2>(a, b, c, lo, hi, tid, nthr, iters);
 }
 
 // ---------------------------------------------------------------- FMA SGEMM

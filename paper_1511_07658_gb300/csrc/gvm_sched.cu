@@ -605,6 +605,96 @@ __device__ __forceinline__ void fma_finish(const SchedParams& p, SchedShared& sh
   }
 }
 
+// Vector tiles on warps 1 .., through the shared memory that the product tiles
+// use. What bounds them is the bytes under way: each thread keeps kVecDepth
+// groups of 32 bytes of its own on their way there (cp.async holds no
+// registers: 66 KB an SM), and reads back only what it copied, so that no
+// thread waits for another. 64 vector adds of 2^22 take 491 us, 714 where the
+// operands are not 16-byte aligned. Loads into registers (eight 16-byte ones of
+// each operand a thread, or single 4-byte ones) took 553 and 5090 us, and more
+// of them spilled, in the product's loop too.
+constexpr int kVecThreads = kFmaThreads - 32;
+constexpr int kVecDepth = 11;
+constexpr uint32_t kVecStage = kVecThreads * 32;  // a's halves, then b's
+static_assert(kVecDepth * kVecStage <= sizeof(FmaSmem), "the groups fit the product tiles' memory");
+
+template <int kBytes>
+__device__ __forceinline__ void cp_async(uint32_t dst, const float* src) {
+  if (kBytes == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// kVec: a, b and c are 16-byte aligned and a group is four consecutive values of
+// each, else every kVecThreads-th. c[i] = a[i] op b[i] for i < len, but for
+// the last len % 4 with kVec.
+template <int OP, bool kVec>
+__device__ __forceinline__ void fma_vector_groups(const float* a, const float* b, float* c, int64_t len, int iters,
+                                                  uint32_t smem) {
+  constexpr int kStep = 4 * kVecThreads;              // values between a thread's groups
+  constexpr int kEach = kVec ? 4 : kVecThreads;       // and between the parts of one
+  constexpr int kBytes = kVec ? 16 : 4;
+  const int t = threadIdx.x - 32;
+  const uint32_t at = smem + t * kBytes;
+  int64_t left = (kVec ? len & ~int64_t(3) : len) - (kVec ? 4 * t : t);  // values from the next group to store on
+  a += kVec ? 4 * t : t;
+  b += kVec ? 4 * t : t;
+  c += kVec ? 4 * t : t;
+  // Copies of the group `ahead` groups after the next one to store.
+  auto issue = [&](int ahead, uint32_t slot) {
+    const int off = ahead * kStep;
+#pragma unroll
+    for (int u = 0; u < (kVec ? 1 : 4); ++u) {
+      if (off + u * kEach < left) {
+        cp_async<kBytes>(slot + u * kEach * kBytes, a + off + u * kEach);
+        cp_async<kBytes>(slot + kVecStage / 2 + u * kEach * kBytes, b + off + u * kEach);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll 1
+  for (int d = 0; d < kVecDepth; ++d) issue(d, at + d * kVecStage);
+  uint32_t slot = at;
+  while (left > 0) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kVecDepth - 1) : "memory");
+    if (kVec) {
+      const uint4 xu = ld_shared_v4(slot), yu = ld_shared_v4(slot + kVecStage / 2);
+      __stcs(reinterpret_cast<float4*>(c),
+             elem_op4<OP>(*reinterpret_cast<const float4*>(&xu), *reinterpret_cast<const float4*>(&yu), iters));
+    } else {
+      float x[4], y[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        x[u] = ld_shared_f32(slot + u * kEach * 4);
+        y[u] = ld_shared_f32(slot + kVecStage / 2 + u * kEach * 4);
+      }
+      const float4 z = elem_op4<OP>(make_float4(x[0], x[1], x[2], x[3]), make_float4(y[0], y[1], y[2], y[3]), iters);
+      const float zs[4] = {z.x, z.y, z.z, z.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u * kEach < left) c[u * kEach] = zs[u];
+    }
+    issue(kVecDepth, slot);  // after the stores: what the slot held is in registers
+    a += kStep;
+    b += kStep;
+    c += kStep;
+    left -= kStep;
+    slot = slot + kVecStage < smem + kVecDepth * kVecStage ? slot + kVecStage : at;
+  }
+}
+
+template <int OP>
+__device__ __forceinline__ void fma_vector(const float* a, const float* b, float* c, int64_t len, int iters,
+                                           uint32_t smem) {
+  const uintptr_t all = reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b) | reinterpret_cast<uintptr_t>(c);
+  if ((all & 15) == 0) {
+    fma_vector_groups<OP, true>(a, b, c, len, iters, smem);
+    const int64_t e = (len & ~int64_t(3)) + threadIdx.x - 32;
+    if (e < len) c[e] = elem_op<OP>(__ldcg(a + e), __ldcg(b + e), iters);
+  } else {
+    fma_vector_groups<OP, false>(a, b, c, len, iters, smem);
+  }
+}
+
 __global__ void __launch_bounds__(kFmaThreads, 2) sched_fma_kernel(const __grid_constant__ SchedParams p) {
   __shared__ SchedShared sh;
   extern __shared__ uint8_t dyn_smem[];
@@ -645,13 +735,12 @@ __global__ void __launch_bounds__(kFmaThreads, 2) sched_fma_kernel(const __grid_
     if (warp == 0) {
       fma_claim(p, sh, nxt, !vec);
     } else if (vec) {
-      const int64_t lo = (int64_t)sh.tile[cur] * b.vadd_tile;
-      const int64_t hi = min(b.n, lo + b.vadd_tile);
-      const float* x = reinterpret_cast<const float*>(b.a);
-      const float* y = reinterpret_cast<const float*>(b.b);
-      float* z = reinterpret_cast<float*>(b.c);
-      if (b.type == kTaskVadd) vadd_range<false, 8>(x, y, z, lo, hi, tid - 32, kFmaThreads - 32);
-      else vmul_range<false, 8>(x, y, z, lo, hi, tid - 32, kFmaThreads - 32, b.k);
+      const int64_t lo = (int64_t)sh.tile[cur] * b.vadd_tile, len = min(b.n - lo, b.vadd_tile);
+      const float* x = reinterpret_cast<const float*>(b.a) + lo;
+      const float* y = reinterpret_cast<const float*>(b.b) + lo;
+      float* z = reinterpret_cast<float*>(b.c) + lo;
+      if (b.type == kTaskVadd) fma_vector<kElemAdd>(x, y, z, len, 0, smem_u32(dyn_smem));
+      else fma_vector<kElemMul>(x, y, z, len, b.k, smem_u32(dyn_smem));
     }
     if (vec) fma_finish(p, sh, cur, kProfVadd);
     else __syncthreads();

@@ -63,3 +63,66 @@ def test_kstep_numbers_are_taken_back(gvm, mode, m, n, k):
         rk.read(18 << 20, v)
         assert np.array_equal(bits(v.numpy()), bits(oracle.vadd(x, y)))
         assert mgr.stats()["device_status"] == 0
+
+
+# The FMA scheduler's vector tiles: 96 threads, groups of four values (16-byte
+# aligned operands) or of every 96th value, eleven groups under way. Lengths
+# around a part, a step of all threads (384), the groups under way and a tile's
+# end; the words around each result must stay as they were.
+@pytest.mark.parametrize("shift", [(0, 0, 0), (1, 0, 0), (0, 2, 0), (0, 0, 3), (3, 1, 2)])
+@pytest.mark.parametrize("op", ["vadd", "vmul"])
+def test_fma_scheduler_vector_groups(gvm, op, shift):
+    sizes = [1, 3, 4, 95, 96, 97, 383, 384, 385, 11 * 384 - 1, 11 * 384, 11 * 384 + 1, 12 * 384 + 5, 1024, 1025, 9999]
+    with gvm.Manager(1, ring_depth=64, sgemm_path="fma", slice_bytes=16 << 20, resident_bytes=12 << 20,
+                     vadd_tile=8192) as mgr:
+        rk = mgr.attach(0)
+        step = 64 << 10
+        jobs = []
+        for i, n in enumerate(sizes):
+            seed = synth.task_seed(5, n)
+            x, y = synth.vadd_inputs(seed, n) if op == "vadd" else synth.vmul_inputs(seed, n)
+            offs = [(3 * i + j) * step + 64 + 4 * s for j, s in enumerate(shift)]
+            rk.write(offs[0], torch.from_numpy(x))
+            rk.write(offs[1], torch.from_numpy(y))
+            rk.write(offs[2] - 16, torch.full((n + 8,), 7.0))
+            jobs.append((n, x, y, offs))
+        for n, _, _, offs in jobs:
+            seq = rk.submit_vadd_resident(*offs, n) if op == "vadd" else rk.submit_vmul_resident(*offs, n, 15)
+        mgr.flush()
+        rk.sync(seq)
+        for n, x, y, offs in jobs:
+            got = torch.empty(n + 8)
+            rk.read(offs[2] - 16, got)
+            got = got.numpy()
+            want = oracle.vadd(x, y) if op == "vadd" else oracle.vmul(x, y, 15)
+            assert np.array_equal(bits(got[4:-4]), bits(want)), n
+            assert np.all(got[:4] == 7.0) and np.all(got[-4:] == 7.0), n
+        assert mgr.stats()["device_status"] == 0
+
+
+# What the split3 scheduler's vector landings took for a result that is not
+# 16-byte aligned must not be slower than for one that is by more than half.
+# (Its stores are 4 bytes a lane; the loads bound it.) The FMA scheduler's
+# groups: three times, for four times the requests.
+@pytest.mark.parametrize("path,most", [("split3", 1.5), ("fma", 3.0)])
+def test_misaligned_vectors_keep_their_rate(gvm, path, most):
+    n, per, ranks = 1 << 20, 8, 8
+    step = 4 * n + 256
+    best = {}
+    with gvm.Manager(ranks, ring_depth=8, sgemm_path=path, slice_bytes=3 * per * step + (1 << 20),
+                     resident_bytes=3 * per * step) as mgr:
+        rks = [mgr.attach(r) for r in range(ranks)]
+        for rk in rks:
+            rk.resident_view(0, (3 * per * step // 4,)).fill_(1.0)
+        torch.cuda.synchronize()
+        for shift in (0, 1):
+            arrays = []
+            for _ in rks:
+                a = (gvm.GvmTask * per)()
+                for i in range(per):
+                    a[i].type, a[i].flags, a[i].n = gvm.GVM_TASK_VADD, gvm.GVM_TASK_RESIDENT, n
+                    a[i].a_off, a[i].b_off, a[i].c_off = 3 * i * step, (3 * i + 1) * step, (3 * i + 2) * step + 4 * shift
+                arrays.append(a)
+            mgr.spmd_run(rks, arrays, 3)
+            best[shift] = min(mgr.spmd_run(rks, arrays, 20)[1])
+    assert best[1] <= most * best[0], best
