@@ -8,7 +8,7 @@ import synth
 
 pytestmark = pytest.mark.gpu
 
-from sgemm_bounds import check_sgemm  # noqa: E402
+from sgemm_bounds import check_sgemm, gamma  # noqa: E402
 
 
 @pytest.fixture(scope="module")
@@ -126,3 +126,40 @@ def test_misaligned_vectors_keep_their_rate(gvm, path, most):
             mgr.spmd_run(rks, arrays, 3)
             best[shift] = min(mgr.spmd_run(rks, arrays, 20)[1])
     assert best[1] <= most * best[0], best
+
+
+# Interior and ragged tiles, rows aligned to 4, 8 and 16 bytes, k below one
+# k-step, several tiles a cluster: the standalone kernel against binary64 by the
+# bound of sgemm_bounds.check_sgemm, and bit for bit the manager's result, whose
+# tiles are 256 (or 192) columns wide where the standalone kernel picks 64 to 256.
+@pytest.mark.parametrize(
+    "shape",
+    [(128, 256, 32), (257, 130, 67), (512, 512, 512), (129, 257, 513), (300, 1001, 77), (130, 260, 100),
+     (1000, 520, 2052), (4096, 2048, 96), (2500, 3000, 40), (256, 256, 1), (768, 1024, 512), (1024, 512, 2048),
+     (520, 512, 256), (200, 300, 96), (384, 640, 44), (1, 257, 31)],
+)
+def test_standalone_kernel_equals_the_manager(gvm, shape):
+    m, n, k = shape
+    A, B = synth.sgemm_inputs(synth.task_seed(13, m % 1000), m, n, k)
+    tA, tB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    C = torch.full((m, n), float("nan"), device="cuda")
+    gvm.sgemm_f32(tA, tB, C, path="split3")
+    torch.cuda.synchronize()
+    R = tA.double() @ tB.double()
+    bound = gamma(k) * (tA.double().abs() @ tB.double().abs()) + k * 2.0 ** -149
+    assert bool(((C.double() - R).abs() <= bound).all())
+    step = [(4 * x + 255) // 256 * 256 for x in (m * k, k * n, m * n)]
+    with gvm.Manager(1, ring_depth=4, sgemm_path="split3", slice_bytes=sum(step) + (1 << 20),
+                     resident_bytes=sum(step)) as mgr:
+        rk = mgr.attach(0)
+        rk.write(0, torch.from_numpy(A))
+        rk.write(step[0], torch.from_numpy(B))
+        seq = rk.submit_sgemm_resident(0, step[0], step[0] + step[1], m, n, k)
+        mgr.flush()
+        rk.sync(seq)
+        out = torch.empty(m, n)
+        rk.read(step[0] + step[1], out)
+        assert np.array_equal(bits(out.numpy()), bits(C.cpu().numpy()))
+    from paper_1511_07658_gb300.manager import kernel_status
+
+    assert kernel_status() == 0
