@@ -132,7 +132,11 @@ typedef struct gvm_config {
   uint64_t idle_poll_ns;    /* sleep of an idle scheduler CTA between polls of the
                                rings; 0 = 1000 ns */
   int32_t grid_ctas;        /* scheduler CTAs; 0 = one per SM (two on the FMA path). The split3
-                               scheduler runs in pairs of CTAs: an odd number is rounded up */
+                               scheduler runs in pairs of CTAs: an odd number is rounded up.
+                               At 0 the scheduler holds every SM: another kernel of the
+                               process waits for the end of its launch, in continuous mode
+                               for gvm_shutdown. Fewer CTAs leave SMs to other kernels
+                               (split3: each pair less leaves two) */
   int32_t ingest_quantum;   /* tasks taken from one rank per ingest pass; 0 = 4 */
   uint64_t copy_run_bytes;  /* host-mode copies of one batch that are adjacent on both
                                sides are merged up to this many bytes; 0 = 16 MiB */
@@ -331,7 +335,11 @@ GVM_API int gvm_task_times(gvm_rank* rank, uint64_t seq, uint64_t* t_ingest_ns, 
    time from the rank's gvm_submit_many call of step i to the moment
    gvm_sync showed task j of that batch complete (ns, CLOCK_MONOTONIC).
    Returns GVM_OK or the first error any rank saw (the remaining steps are
-   skipped). The batch submit call counts as each of its tasks' submit. */
+   skipped). The batch submit call counts as each of its tasks' submit.
+   The threads of ranks 1 .. nranks - 1 (rank 0 runs on the caller's) belong to
+   the manager and are kept between calls of this and the three below: after
+   a run they look for the next for 100 us, then sleep; gvm_shutdown ends
+   them. GVM_ENOMEM, with nothing run, when one cannot be created. */
 GVM_API int gvm_spmd_run(gvm_ctx* ctx, gvm_rank* const* ranks, const gvm_task* const* tasks,
                          const uint32_t* counts, int32_t nranks, int32_t steps, float* step_ms_device,
                          float* launch_ms_device, double* step_ms_host, double* const* latency_ns);

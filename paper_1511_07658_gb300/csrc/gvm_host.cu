@@ -794,14 +794,13 @@ void fill_body(gvm_ctx* ctx, gvm_rank* r, const Prep& p, uint64_t seq, uint64_t 
                                              t->m, t->n, t->k, &body->tmA, &body->tmB);
       tm = 256;
       tn = pair_tile_n(maps);
-      body->flags |= kFlagSplit3 | kFlagTmA * maps;
+      body->flags |= kFlagTmA * maps;
       body->vadd_tile = tn;
     }
     body->tiles_m = (uint32_t)((t->m + tm - 1) / tm);
     body->tiles_n = (uint32_t)((t->n + tn - 1) / tn);
     body->ntiles = body->tiles_m * body->tiles_n;
   }
-  body->nsplit = 0;
 }
 
 // Admits tasks[0 .. count-1] of rank r in order, as far as the ring and the

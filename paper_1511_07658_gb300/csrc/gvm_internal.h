@@ -22,7 +22,6 @@ enum : uint32_t { kTaskVadd = 1, kTaskSgemm = 2, kTaskVmul = 3 };
 enum : uint32_t {
   kFlagNeedsReady = 1u,   // host-mode inputs: wait for the input stream's ready word
   kFlagNeedsD2H = 2u,     // host-mode output: the output stream copies and completes
-  kFlagSplit3 = 4u,       // SGEMM on the split-bf16 tensor-core path
   kFlagDirectOut = 8u,    // host-mode output written by the kernel into host memory
   kFlagTmA = 16u,         // split3: tmA maps A (ingest copies it)
   kFlagTmB = 32u,         // split3: tmB maps B (ingest copies it)
@@ -37,8 +36,7 @@ enum : uint32_t {
   kStatusBadTask = 2,
 };
 enum : uint32_t {
-  kWhereReadyWait = 1,
-  kWhereSplitWait = 2,
+  kWhereReadyWait = 1,  // 2 is not used
   kWhereFullBarrier = 3,
   kWhereEmptyBarrier = 4,
   kWhereAccumBarrier = 5,
@@ -46,8 +44,6 @@ enum : uint32_t {
   kWhereItemWait = 7,   // a warp waiting for its CTA's next claimed tile
   kWhereItemRing = 8,   // the claiming warp waiting for a free item slot
 };
-
-constexpr uint32_t kClaimLocked = 0x40000000u;  // claim counter while a slot is rewritten
 
 // ---- task body: written by the host into its ring, copied by the device ----
 // 384 bytes; the two tensor maps must stay 64-byte aligned (they are at 0, 128).
@@ -59,30 +55,27 @@ struct alignas(128) TaskBody {
   uint32_t rank;
   uint32_t slot;
   uint32_t tag;      // (seq + 1) truncated to 32 bits; never 0
-  uint32_t ntiles;   // all tiles of the task (split + main)
-  uint32_t nsplit;   // split tiles (split3 only)
+  uint32_t ntiles;   // all tiles of the task
+  uint32_t pad0;
   uint32_t tiles_m;
   uint32_t tiles_n;
-  uint32_t kp;       // k rounded up to a multiple of 8 (split3 scratch row pitch)
+  uint32_t pad1;
   int32_t m;
   int32_t k;
   int64_t n;
   int64_t vadd_tile; // elements per vector-add tile; split3 SGEMM: columns per tile
   uint64_t a, b, c;  // device addresses of the operands
-  uint64_t scratch;  // device address of the split3 planes (A planes, then B^T planes)
-  uint64_t scratch_b;// device address of the B^T planes
-  uint64_t pad[3];
+  uint64_t pad2[5];
 };
 static_assert(sizeof(TaskBody) == 384, "TaskBody layout");
 
 // Device task table entry: the body plus its counters on their own line.
 struct alignas(128) DevTask {
   TaskBody body;
-  uint32_t claimed[2];   // tiles claimed per phase
   uint32_t tiles_done;
-  uint32_t split_done;
-  uint64_t t_ingest;     // globaltimer when taken from the ring
-  uint32_t pad2[26];
+  uint32_t pad;
+  uint64_t t_ingest;  // globaltimer when taken from the ring
+  uint32_t pad2[28];
 };
 static_assert(sizeof(DevTask) == 512, "DevTask layout");
 

@@ -239,9 +239,11 @@ extern "C" int gvm_sgemm_f32(const float* A, const float* B, float* C, int32_t m
   const int pairs = sms / 2;
   // Columns per tile: the fewest waves of tiles weighted by a tile's time. A
   // k-step of 256 x n costs about 256 + n units (A's share of the staging
-  // does not shrink with n): measured, with three landings, 15 / 17 / 18 / 21
-  // us at 512^3 (16, 8, 6 and 4 tiles of 76 pairs; 64 columns taken), 108 / 64
-  // / 70 / 44 us at 2048^3 (256, 128, 88 and 64 tiles; 256 taken, 41 us now).
+  // does not shrink with n). Measured, one launch from a cold L2, at 64 / 128 /
+  // 192 / 256 columns: 512^3 16.4 / 16.4 / 18.4 / 20.5 us (64 taken), 2048^3
+  // 107 / 64 / 68 / 43 (256 taken). Packed operands, 64 / 128 / 192: 1530 x 1027
+  // x 2001 94 / 61 / 68 (128 taken), 2047^3 168 / 104 / 115 (128), 4095^3 1077 /
+  // 584 / 487 (192).
   CUtensorMap tmA, tmB;
   memset(&tmA, 0, sizeof(tmA));
   memset(&tmB, 0, sizeof(tmB));

@@ -219,8 +219,7 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t saddr, uint32_t rank) {
 // ordering this CTA's own accesses only (CTA-scope release): what the waiter
 // goes on to do is issue MMAs, which read each CTA's shared memory in place. A
 // cluster-scope release would also wait for all of the thread's earlier
-// accesses to be performed cluster-wide: about 1000 clocks a k-step (2048^3
-// in 56 us instead of 35).
+// accesses to be performed cluster-wide: about 1000 clocks a k-step.
 __device__ __forceinline__ void mbar_arrive_cta(uint64_t* bar, uint32_t rank) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(mapa_shared(smem_u32(bar), rank)) : "memory");
 }

@@ -15,7 +15,7 @@
  *            "timed": after it, inside the first phase's timed region
  *            (T_init of Eq. 1; the first phase must then copy)
  *   PHASE    PATH:MODE, run in order, each on its own start signal:
- *            PATH  GVM_SGEMM_* path number (0 = FMA, 2 = split3 fused)
+ *            PATH  GVM_SGEMM_* path number (0 = FMA, 2 = split3)
  *            MODE  resident  operands copied to the device before the
  *                            first start; per task kernel + synchronize
  *                  copy      per task: copy A and B in, kernel, copy C out

@@ -226,7 +226,7 @@ __device__ __forceinline__ IngestOut ingest_pass(const SchedParams& p, uint64_t*
           const uint32_t idx = r * p.depth + ((t + base + i) & (p.depth - 1));
           const uint4* src = reinterpret_cast<const uint4*>(&p.host_desc[idx]) + kFieldsAt / 16;
           h0[i] = ld_volatile_v4(src);      // type, flags, rank, slot
-          h1[i] = ld_volatile_v4(src + 1);  // tag, ntiles, nsplit, tiles_m
+          h1[i] = ld_volatile_v4(src + 1);  // tag, ntiles
           rdy[i] = ld_relaxed_gpu(&p.ready[idx]);
         }
       }
@@ -760,10 +760,12 @@ __global__ void __launch_bounds__(kFmaThreads, 2) sched_fma_kernel(const __grid_
 // every role of both walks the items in order. A GEMM tile is the pair's: the
 // CTAs stage their halves of the operands, the leader issues the MMAs, each
 // CTA's epilogue warps store its 128 rows. A vector tile is split in two
-// halves, each run by a CTA's converter and epilogue warps. Either way each
-// CTA counts its half, so a task is complete after 2 x ntiles counts. The
-// peer's control warp hands read items back to the leader. No warp
-// waits for another warp's tile except through the pipeline's barriers.
+// halves, each run by a CTA's converter warps from the landing ring (by
+// converter and epilogue warps together where bulk copies cannot address the
+// operands). Either way each CTA counts its half, so a task is complete after
+// 2 x ntiles counts. The peer's control warp hands read items back to the
+// leader. No warp waits for another warp's tile except through the pipeline's
+// barriers.
 
 constexpr int kItems = 4;                               // items in flight between the control warp and the others
 constexpr uint32_t kItemExit = 0, kItemNop = 0xffu;     // besides the task types
@@ -777,13 +779,13 @@ struct alignas(16) PrItem {
   uint32_t tile;
   uint32_t first;  // SGEMM: number of the tile's first k-step (gvm_ring.h)
   uint32_t type, flags, rank, slot;
-  uint32_t tag, ntiles, nsplit, tiles_m;
-  uint32_t tiles_n, kp;
+  uint32_t tag, ntiles, pad0, tiles_m;
+  uint32_t tiles_n, pad1;
   int32_t m;
   int32_t k;
   int64_t n;
   int64_t span;  // vector tasks: elements per tile; SGEMM: columns per tile
-  uint64_t a, b, c, scratch;
+  uint64_t a, b, c, pad2;
 };
 constexpr int kItemFields = 6;  // 16-byte pieces of task fields
 constexpr int kItemFieldK = 2;  // the one that ends with k
@@ -791,13 +793,12 @@ static_assert(offsetof(TaskBody, k) == kFieldsAt + 16 * kItemFieldK + 12, "k's p
 static_assert(sizeof(PrItem) == 16 * (kItemFields + 1) && offsetof(TaskBody, c) - offsetof(TaskBody, type) ==
                   offsetof(PrItem, c) - offsetof(PrItem, type), "item = header + task fields");
 
-// One thread: ask L2 for a GEMM item's task operands -- A's block of tile_m rows
+// One thread: ask L2 for a GEMM item's task operands -- A's block of kPrM rows
 // of the tile's row (from the tile in column 0 of its row) and all of B
 // (from tile (0, 0)) -- so that each task's operands are requested once, in
 // pieces of at most 1 MiB, when they are 16-byte aligned, span a multiple
 // of 16 bytes and B holds at most 4 MiB. A hint only.
-template <class Item>
-__device__ __forceinline__ void prefetch_task_operands(const Item& it, int64_t tile_m) {
+__device__ __forceinline__ void prefetch_task_operands(const PrItem& it) {
   if (it.kind != kTaskSgemm || (it.k & 3) || ((it.a | it.b) & 15)) return;
   const uint32_t tm = it.tile / it.tiles_n, tn = it.tile % it.tiles_n;
   if (tn != 0) return;
@@ -807,8 +808,8 @@ __device__ __forceinline__ void prefetch_task_operands(const Item& it, int64_t t
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(addr + off), "r"((uint32_t)len) : "memory");
     }
   };
-  const int64_t rows = min(tile_m, (int64_t)it.m - (int64_t)tm * tile_m);
-  if (rows > 0) pf(it.a + (uint64_t)tm * (uint64_t)tile_m * (uint64_t)it.k * 4u, (uint64_t)rows * (uint64_t)it.k * 4u);
+  const int64_t rows = min((int64_t)kPrM, (int64_t)it.m - (int64_t)tm * kPrM);
+  if (rows > 0) pf(it.a + (uint64_t)tm * kPrM * (uint64_t)it.k * 4u, (uint64_t)rows * (uint64_t)it.k * 4u);
   const uint64_t b_bytes = (uint64_t)it.k * (uint64_t)it.n * 4u;
   if (tm == 0 && b_bytes <= (4u << 20) && (b_bytes & 15) == 0) pf(it.b, b_bytes);
 }
@@ -936,7 +937,7 @@ PAIR_ROLE pair_control(const SchedParams& p, PairSchedShared& sh) {
       sh.prof[kProfAcquire] += globaltimer() - t0;
       // L2 prefetch, a few tiles ahead of the producers: the item two claims
       // back (its slot is rewritten only two claims from now).
-      if (p.prefetch && seq >= 2) prefetch_task_operands(sh.items[(seq + 2) % kItems], kPrM);
+      if (p.prefetch && seq >= 2) prefetch_task_operands(sh.items[(seq + 2) % kItems]);
     }
     __syncwarp();
     if (got == 0) break;
