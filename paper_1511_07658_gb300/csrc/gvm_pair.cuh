@@ -482,8 +482,7 @@ __device__ __forceinline__ bool pr_convert_aligned(const PrTile t, uint32_t land
   const int slabs = t.ncols >> 6;
   const bool has_a = t.row0 + (int)ps->cta * 128 < t.m;
   const uint32_t r = (uint32_t)lane >> 2, c = (uint32_t)lane & 3u;
-  const uint32_t rd0 = (uint32_t)w * 1024u + r * 128u + (((2u * c) ^ r) << 4);
-  const uint32_t rd1 = (uint32_t)w * 1024u + r * 128u + (((2u * c + 1u) ^ r) << 4);
+  const uint32_t rd0 = (uint32_t)w * 1024u + r * 128u + (((2u * c) ^ r) << 4);  // and the next chunk at rd0 ^ 16
   const uint32_t wr = swz64(r, c);
   for (int kb = (int)((it + (uint32_t)par) & 1u); kb < nkb; kb += 2) {
     const uint32_t q = it + (uint32_t)kb, ql = it_l + (uint32_t)kb;
@@ -499,7 +498,7 @@ __device__ __forceinline__ bool pr_convert_aligned(const PrTile t, uint32_t land
     auto read_b = [&](int b) {
       if (b < slabs) {
         xb[b][0] = ld_shared_v4(ld + kPrLandA + (uint32_t)b * kPrSlab + rd0);
-        xb[b][1] = ld_shared_v4(ld + kPrLandA + (uint32_t)b * kPrSlab + rd1);
+        xb[b][1] = ld_shared_v4(ld + kPrLandA + (uint32_t)b * kPrSlab + (rd0 ^ 16u));
       }
     };
     auto put = [&](const uint4 (&x)[2], uint32_t hi_at, uint32_t lo_at) {
@@ -515,7 +514,7 @@ __device__ __forceinline__ bool pr_convert_aligned(const PrTile t, uint32_t land
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         xa[j][0] = ld_shared_v4(ld + (uint32_t)j * 4096u + rd0);
-        xa[j][1] = ld_shared_v4(ld + (uint32_t)j * 4096u + rd1);
+        xa[j][1] = ld_shared_v4(ld + (uint32_t)j * 4096u + (rd0 ^ 16u));
       }
     }
     read_b(0);
