@@ -16,7 +16,7 @@
 // bf16 ring (kPrStages) decouples the conversion from the MMAs. Aligned
 // operands are read into registers before the stage is awaited. With three
 // landings of 35 KB and the stage awaited first, 1024 products of 512^3 took
-// 0.80 ms (now 0.74), the grouped mix 2.23 (2.01), 2048^3 43 us (40.5) and 64
+// 0.80 ms (now 0.74), the grouped mix 2.23 (2.01), 2048^3 43 us (39) and 64
 // vector adds of 4 M values 0.55 ms (0.50).
 //
 // CTA roles (kPrThreads = 480, one CTA per SM):
