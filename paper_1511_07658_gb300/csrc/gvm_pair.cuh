@@ -252,9 +252,11 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
   }
 }
 // The same waits by all lanes of a converged warp, left by all of them
-// together: what follows may be warp-collective (tcgen05.ld, shuffles).
+// together: what follows may be warp-collective (tcgen05.ld, shuffles). The
+// limit comes by reference, to be read once a wait goes on and not held through
+// the converters' loops.
 template <bool kCluster>
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, uint64_t timeout_ns,
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, const uint64_t& timeout_ns,
                                                volatile uint32_t* cta_abort) {
   auto done = [&]() -> bool {
     const bool ok = kCluster ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity);
@@ -450,14 +452,14 @@ __device__ __forceinline__ float ld_shared_f32(uint32_t addr) {
 // Converter warps, landing ql: its operands have landed. Landings also serve
 // vector tiles, so that ql runs ahead of the k-step's number q, by an even
 // number: both belong to the same group.
-__device__ __forceinline__ bool pr_wait_landed(PrShared* ps, uint32_t ql, uint64_t timeout_ns, uint32_t* cta_abort,
+__device__ __forceinline__ bool pr_wait_landed(PrShared* ps, uint32_t ql, const uint64_t& timeout_ns, uint32_t* cta_abort,
                                                uint32_t* fail_where) {
   if (mbar_wait_warp<false>(&ps->landed[ql % kPrLand], (ql / kPrLand) & 1u, timeout_ns, cta_abort)) return true;
   if ((threadIdx.x & 31) == 0) pr_fail(ps, cta_abort, fail_where, kWhereEmptyBarrier);
   return false;
 }
 // Converter warps, k-step q: the MMAs have read its stage's previous k-step, q - 3.
-__device__ __forceinline__ bool pr_wait_stage(PrShared* ps, uint32_t q, uint64_t timeout_ns, uint32_t* cta_abort,
+__device__ __forceinline__ bool pr_wait_stage(PrShared* ps, uint32_t q, const uint64_t& timeout_ns, uint32_t* cta_abort,
                                               uint32_t* fail_where) {
   if (!pr_stage_used(q) || mbar_wait_warp<false>(&ps->empty[pr_empty_bar(q - kPrStages)], pr_empty_parity(q - kPrStages),
                                                  timeout_ns, cta_abort))
@@ -474,7 +476,7 @@ __device__ __forceinline__ bool pr_wait_stage(PrShared* ps, uint32_t q, uint64_t
 // is never stored). Returns false when a wait ran out.
 // Both operands aligned:
 __device__ __forceinline__ bool pr_convert_aligned(const PrTile t, uint32_t land0, uint32_t st0, PrShared* ps,
-                                                   uint32_t it, uint32_t it_l, uint64_t timeout_ns,
+                                                   uint32_t it, uint32_t it_l, const uint64_t& timeout_ns,
                                                    uint32_t* cta_abort, uint32_t* fail_where) {
   const int cw = (int)(threadIdx.x >> 5) - kPrConvWarp0, lane = threadIdx.x & 31;
   const int par = cw / kPrGroupWarps, w = cw % kPrGroupWarps;
@@ -554,7 +556,7 @@ __device__ __forceinline__ bool pr_convert_aligned(const PrTile t, uint32_t land
 // atoms at a time, so that the loop needs no more registers than the aligned
 // one.
 __device__ __forceinline__ bool pr_convert_packed(const PrTile t, uint32_t land0, uint32_t st0, PrShared* ps, uint32_t it,
-                                               uint32_t it_l, uint64_t timeout_ns, uint32_t* cta_abort,
+                                               uint32_t it_l, const uint64_t& timeout_ns, uint32_t* cta_abort,
                                                uint32_t* fail_where) {
   const int cw = (int)(threadIdx.x >> 5) - kPrConvWarp0, lane = threadIdx.x & 31;
   const int par = cw / kPrGroupWarps, w = cw % kPrGroupWarps;
@@ -670,7 +672,7 @@ __device__ __forceinline__ bool pr_convert_packed(const PrTile t, uint32_t land0
 }
 
 __device__ __forceinline__ bool pr_convert(const PrTile t, uint8_t* land, uint8_t* stages, PrShared* ps, uint32_t it,
-                                           uint32_t it_l, uint64_t timeout_ns, uint32_t* cta_abort,
+                                           uint32_t it_l, const uint64_t& timeout_ns, uint32_t* cta_abort,
                                            uint32_t* fail_where) {
   const uint32_t land0 = smem_u32(land), st0 = smem_u32(stages);
   if (t.land == (kPrMapA | kPrMapB))
@@ -733,12 +735,10 @@ __device__ __forceinline__ bool pr_vec_produce(const float* a, const float* b, i
   return true;
 }
 
-// Converter warps: c = a op b over the landings of this warp's group. Whole
-// landings run unrolled. A function of its own: inlined into the converters'
-// role, its code changed with the product loops beside it (64 vector adds of
-// 2^22 493 to 507 us a launch, multiplies 593 to 630; now 496 and 555).
+// Converter warps: c = a op b over the landings of this warp's group; whole
+// landings run unrolled (64 vector multiplies of 2^22 593 to 540 us a launch).
 template <int OP>
-static __device__ __noinline__ bool pr_vec_convert(const float* a, const float* b, float* c, int64_t len, int iters,
+__device__ __forceinline__ bool pr_vec_convert(const float* a, const float* b, float* c, int64_t len, int iters,
                                                uint8_t* land, PrShared* ps, uint32_t it_l, uint64_t timeout_ns,
                                                uint32_t* cta_abort, uint32_t* fail_where) {
   const int cw = (int)(threadIdx.x >> 5) - kPrConvWarp0, lane = threadIdx.x & 31;
