@@ -147,7 +147,8 @@ typedef struct gvm_config {
                                rank's output stream (Section 5's data path); 1 = the
                                scheduler writes it straight into c through the buffer's
                                device mapping (page-locked memory the GPU can address;
-                               a buffer without one uses the staged path), so outputs
+                               a buffer without one, or not 4-byte aligned, uses the
+                               staged path), so outputs
                                take no staging and no copy */
   int32_t l2_prefetch;      /* split3: 1 = the claiming warp asks L2 for each task's operands
                                (bulk prefetch, a few tiles ahead; a hint, no result depends

@@ -732,7 +732,8 @@ int prep_task(gvm_rank* r, const gvm_task* t, Prep* p) {
   p->bytes_c = bytes_c;
   p->c_direct = 0;
   p->out_pageable = !resident && bytes_c > 0 && p_kc == 0 && !stream_mode(r->ctx);
-  if (!resident && bytes_c > 0 && p_kc == 1 && r->ctx->cfg.direct_output && !stream_mode(r->ctx)) {
+  if (!resident && bytes_c > 0 && p_kc == 1 && r->ctx->cfg.direct_output && !stream_mode(r->ctx) &&
+      (reinterpret_cast<uintptr_t>(t->c) & 3) == 0) {  // the kernels store floats: other addresses are copied to
     // The buffer's device mapping (the same address under unified addressing).
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, t->c) == cudaSuccess && at.devicePointer != nullptr)

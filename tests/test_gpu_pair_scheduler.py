@@ -163,3 +163,26 @@ def test_standalone_kernel_equals_the_manager(gvm, shape):
     from paper_1511_07658_gb300.manager import kernel_status
 
     assert kernel_status() == 0
+
+
+# A host result buffer off a 4-byte boundary is not one the kernel can store to:
+# with direct output it takes the staged path, and the bytes around it stay.
+@pytest.mark.parametrize("path", ["split3", "fma"])
+@pytest.mark.parametrize("offset", [1, 2, 3, 4])
+def test_direct_output_to_any_byte_address(gvm, path, offset):
+    n = 5001
+    x, y = synth.vadd_inputs(synth.task_seed(6, offset), n)
+    a, b = torch.from_numpy(x).pin_memory(), torch.from_numpy(y).pin_memory()
+    out = torch.full((4 * n + 16,), 0x5A, dtype=torch.uint8).pin_memory()
+    with gvm.Manager(1, ring_depth=4, sgemm_path=path, slice_bytes=8 << 20, direct_output=True) as mgr:
+        rk = mgr.attach(0)
+        t = gvm.GvmTask()
+        t.type, t.n = gvm.GVM_TASK_VADD, n
+        t.a, t.b, t.c = a.data_ptr(), b.data_ptr(), out.data_ptr() + offset
+        seq = rk.submit(t)
+        mgr.flush()
+        rk.sync(seq)
+        got = out.numpy()
+        assert np.array_equal(got[offset:offset + 4 * n].copy().view(np.uint32), bits(oracle.vadd(x, y)))
+        assert np.all(got[:offset] == 0x5A) and np.all(got[offset + 4 * n:] == 0x5A)
+        assert mgr.stats()["device_status"] == 0
